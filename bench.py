@@ -89,7 +89,7 @@ def pinned_lp(lp):
 
 def kernel_source_sha() -> str:
     h = hashlib.sha256()
-    for f in ("pdlp_kernels.cu", "pdlp_internal.cuh"):
+    for f in ("pdlp_kernels.cu", "pdlp_step.cuh", "pdlp_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2311_12180_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -896,6 +896,8 @@ def main():
         cpu = cpu_baseline(lp)
 
     kernels_per_period = 2 * (period + max(4, period // 8)) + 4  # + check_primal, infeas, check_dual, restart
+    if lay["K_stored"] + lay["KT_stored"] + 8 * (lp.m + lp.n) <= 8_000_000:
+        kernels_per_period = 1  # a small LP's period is one launch
     line = {
         "metric": METRIC,
         "value": value,

@@ -18,7 +18,7 @@
  * diagonal preconditioning of Sec. 2.2 (done on the GPU at create time), and
  * termination on the relative KKT error of the ORIGINAL problem (Sec. 4.1).
  * Every step of the iteration runs in this library's CUDA kernels on one GPU;
- * the host only launches CUDA graphs and polls a status word.
+ * the host only enqueues check periods and polls a status word.
  *
  * Conventions for every function below:
  *   - Return value: PDLP_OK (0) or a negative PDLP_ERR_* code.  No function
@@ -106,7 +106,7 @@ typedef struct {
   double omega, eta_hat;  /* primal weight and next trial step size (scaled LP) */
   double setup_ms;        /* pdlp_create device work (transfer + transpose + scaling) */
   double solve_ms;        /* wall time of the last solve call */
-  int64_t graph_launches; /* CUDA-graph launches in the last solve */
+  int64_t graph_launches; /* check periods enqueued in the last solve */
   int64_t f64_switch_iter; /* value_bits = 32 only: k at which the steps moved to FP64 K, -1 never */
   /* infeasible statuses only (else 0), on the original LP: PDLP_PRIMAL_INFEASIBLE: ray_obj =
      q'yr + l'lambda+ - u'lambda-, ray_res = ||(-K'yr - lambda, min(yr_G, 0))||_2;
@@ -214,7 +214,7 @@ int pdlp_solve_warm(pdlp_solver *s, const double *x0, const double *y0, double t
 /* Non-blocking pieces of pdlp_solve, for callers that overlap work or time
  * the iteration:  pdlp_begin resets the state (warm point as in
  * pdlp_solve_warm, NULLs = cold) and evaluates KKT(z^{0,0});
- * pdlp_run_periods enqueues n_periods CUDA-graph launches (each covers P
+ * pdlp_run_periods enqueues n_periods check periods (each covers P
  * accepted steps plus one restart / termination check, or stops early once
  * the solve has ended) without waiting; pdlp_poll waits for the enqueued work
  * and returns the status (-1 = still running); pdlp_finish writes the outputs
@@ -256,11 +256,12 @@ int pdlp_get_state(const pdlp_solver *s, void *buf, size_t cap, size_t *bytes);
 int pdlp_set_state(pdlp_solver *s, const void *buf, size_t bytes);
 int pdlp_resume(pdlp_solver *s, double *x_out, double *y_out, int *status, int64_t *iters);
 
-/* Enqueues n_periods periods like pdlp_run_periods but launches each kernel
- * directly (no graph) between CUDA events on the solver's stream, then waits
- * and adds each kernel class's event-measured device time to ms[i] and its
- * launch count to launches[i] (arrays of pdlp_kernel_count() entries, caller
- * zeroes them).  Same arithmetic as the graph path. */
+/* Runs n_periods periods like pdlp_run_periods but as single step and check
+ * kernels (also where a period is one launch), each between CUDA events on
+ * the solver's stream, then waits and adds each kernel class's event-measured
+ * device time to ms[i] and its launch count to launches[i] (arrays of
+ * pdlp_kernel_count() entries, caller zeroes them).  The results are those of
+ * pdlp_run_periods, bit for bit. */
 int pdlp_time_kernels(pdlp_solver *s, int32_t n_periods, double *ms, int64_t *launches);
 int32_t pdlp_kernel_count(void);
 const char *pdlp_kernel_name(int32_t i);

@@ -2,9 +2,10 @@
 // validation, the sliced-ELL layout of K and K' (host, once per LP: the
 // internal row order and the work items), the transpose of K, Sec. 2.2
 // scaling and the sliced-ELL copies on the device, and the
-// solve driver that replays a captured CUDA graph of one check period and
-// polls a pinned copy of the device state one period behind, so the GPU never
-// waits for the host.
+// solve driver that launches one check period after another (one kernel for
+// small LPs, pdlp_period.cu, else a captured CUDA graph) and polls a pinned
+// copy of the device state one period behind, so the GPU never waits for the
+// host.
 
 #include <cuda_runtime.h>
 
@@ -89,6 +90,9 @@ struct pdlp_solver {
   double *c = nullptr, *q = nullptr, *l = nullptr, *u = nullptr, *l0 = nullptr, *u0 = nullptr;
   int gridA = 1, gridB = 1, gridR1 = 1, gridR2 = 1, gridR3 = 1, gridI = 1;
   int slots = 0;
+  PeriodPlan period;             // ctas > 0: a check period is one launch (pdlp_period.cu), else the graph below
+  bool ready = false;            // a period can be enqueued
+  PeriodSync *h_sync = nullptr;  // pinned
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -192,13 +196,17 @@ void free_solver(pdlp_solver *s) {
   if (s->h_st) cudaFreeHost(s->h_st);
   if (s->h_poll) cudaFreeHost(s->h_poll);
   if (s->h_scal) cudaFreeHost(s->h_scal);
+  if (s->h_sync) cudaFreeHost(s->h_sync);
   if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }
 
+// What enqueueing a period needs: nothing for a one-launch period, else the
+// CUDA graph of one check period.
 int build_graph(pdlp_solver *s) {
-  if (s->gexec) return PDLP_OK;
+  s->ready = true;
+  if (s->period.ctas || s->gexec) return PDLP_OK;
   CK(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < s->slots && e == cudaSuccess; ++i) {
@@ -219,6 +227,13 @@ int build_graph(pdlp_solver *s) {
   s->graph = g;
   CK(cudaGraphInstantiate(&s->gexec, s->graph, 0));
   return PDLP_OK;
+}
+
+// Enqueues one check period.
+cudaError_t enqueue_period(pdlp_solver *s) {
+  s->launches++;
+  if (s->period.ctas) return launch_period(s->period, s->K, s->KT, s->V, s->st, s->slots, s->stream);
+  return cudaGraphLaunch(s->gexec, s->stream);
 }
 
 int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const double *c, const int32_t *row_ptr,
@@ -322,6 +337,7 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   CKS(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, s->device));
   CKS(cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->device));
   CKS(kernels_init());
+  CKS(period_init());
   if (stream) {
     s->stream = (cudaStream_t)stream;
   } else {
@@ -334,6 +350,7 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   CKS(cudaMallocHost((void **)&s->h_st, sizeof(DevState)));
   CKS(cudaMallocHost((void **)&s->h_poll, 2 * sizeof(DevState)));
   CKS(cudaMallocHost((void **)&s->h_scal, 8 * sizeof(double)));
+  CKS(cudaMallocHost((void **)&s->h_sync, sizeof(PeriodSync)));
   std::memset(s->h_st, 0, sizeof(DevState));
   s->h_st->status = ST_RUNNING;
 
@@ -377,6 +394,7 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   const size_t o_sc = L.take(8 * (8 + scalars_work_doubles()));
   const long long npw = 1LL << 20;  // exponent factors for the first 2^20 steps (16 MB)
   const size_t o_pw = L.take(16 * (size_t)npw);
+  const size_t o_ps = L.take(sizeof(PeriodSync)), o_pp = L.take(8 * period_part_doubles());
   s->arena_bytes = L.off;
   CKS(cudaMalloc((void **)&s->arena, s->arena_bytes));
   char *A = s->arena;
@@ -451,6 +469,8 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   V.trace = (TraceRec *)(A + o_tr);
   V.pw = (const double *)(A + o_pw);
   V.npw = npw;
+  s->period.sync = (PeriodSync *)(A + o_ps);
+  s->period.part = (double *)(A + o_pp);
   V.perm_r = s->perm_r;
   V.perm_c = s->perm_c;
 
@@ -566,11 +586,14 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
                    (const double *)(B + o_kv), f32 ? (const float *)(B + o_kf) : nullptr};
     s->KT = SellMat{n, (int32_t)LT.items.size(), (const int4 *)(B + o_tit), (const int32_t *)(B + o_ti),
                     (const double *)(B + o_tv), f32 ? (const float *)(B + o_tf) : nullptr};
-    // the solve's CUDA graph (one check period) is captured and instantiated
-    // now, on the host, while the device is still scaling: it needs only the
+    // how a check period runs is decided, and the CUDA graph of the step
+    // kernels, where it is they, is captured and instantiated now, on the host, while the device is still scaling: it needs only the
     // pointers and grids, all known here
     s->slots = prm.check_period + (prm.check_period / 8 > 4 ? prm.check_period / 8 : 4);
     {
+      s->period.grids = PeriodGrids{s->gridA, s->gridB, s->gridR1, s->gridR2, s->gridI, s->gridR3};
+      period_plan(s->period, m, n, LK.items.data(), (int)LK.items.size(), LT.items.data(), (int)LT.items.size(),
+                  LK.total + LT.total, f32 ? 4 : 8, s->num_sms);
       const int grc = build_graph(s);
       if (grc) {
         free_solver(s);
@@ -768,8 +791,12 @@ int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, i
   h.eps_infeas = s->V.qd ? 0.0 : s->prm.eps_infeas;  // the certificates are the LP's
   CK(cudaMemcpyAsync(s->st, s->h_st, sizeof(DevState), cudaMemcpyHostToDevice, st));
   // KKT(z^{0,0}): K'y, Kx and the pieces of eq. (kkt) at the start point
-  CK(launch_check_primal(s->KT, V, s->st, s->gridR1, st));
-  CK(launch_check_dual(s->K, V, s->st, s->gridR2, st));
+  if (s->period.ctas) {
+    CK(launch_period(s->period, s->K, s->KT, V, s->st, 0, st));
+  } else {
+    CK(launch_check_primal(s->KT, V, s->st, s->gridR1, st));
+    CK(launch_check_dual(s->K, V, s->st, s->gridR2, st));
+  }
   s->launches = 0;
   s->have_result = false;
   s->last_status = ST_RUNNING;
@@ -779,12 +806,9 @@ int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, i
 
 int pdlp_run_periods(pdlp_solver *s, int32_t n_periods) {
   g_err.clear();
-  if (!s || !s->gexec) return fail(PDLP_ERR_INVALID, "call pdlp_begin first");
+  if (!s || !s->ready) return fail(PDLP_ERR_INVALID, "call pdlp_begin first");
   CK(cudaSetDevice(s->device));
-  for (int32_t i = 0; i < n_periods; ++i) {
-    CK(cudaGraphLaunch(s->gexec, s->stream));
-    s->launches++;
-  }
+  for (int32_t i = 0; i < n_periods; ++i) CK(enqueue_period(s));
   return PDLP_OK;
 }
 
@@ -808,7 +832,15 @@ int pdlp_finish(pdlp_solver *s, double *x_out, double *y_out, int *status, int64
   CK(cudaMemcpyAsync(s->h_st, s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
   if (x_out) CK(cudaMemcpyAsync(x_out, s->V.xout, 8 * (size_t)s->n, cudaMemcpyDeviceToHost, st));
   if (y_out && s->m) CK(cudaMemcpyAsync(y_out, s->V.yout, 8 * (size_t)s->m, cudaMemcpyDeviceToHost, st));
+  s->h_sync->error = 0;
+  if (s->period.ctas && !s->period.cluster)
+    CK(cudaMemcpyAsync(s->h_sync, s->period.sync, sizeof(PeriodSync), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (s->h_sync->error) {
+    CK(cudaMemsetAsync(s->period.sync, 0, sizeof(PeriodSync), st));
+    CK(cudaStreamSynchronize(st));
+    return fail(PDLP_ERR_CUDA, "a check period timed out at its grid barrier; the results are incomplete");
+  }
   s->solve_ms = now_ms() - s->t0;
   s->have_result = true;
   s->last_status = s->h_st->status;
@@ -825,14 +857,12 @@ static int drive(pdlp_solver *s, double *x_out, double *y_out, int *status, int6
   const double limit_ms = s->prm.time_limit_s > 0.0 ? 1000.0 * s->prm.time_limit_s : INFINITY;
   // one period in flight ahead of the one being polled
   int slot = 0;
-  CK(cudaGraphLaunch(s->gexec, st));
-  s->launches++;
+  CK(enqueue_period(s));
   CK(cudaMemcpyAsync(&s->h_poll[slot], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
   CK(cudaEventRecord(s->ev[slot], st));
   for (;;) {
     const int nxt = slot ^ 1;
-    CK(cudaGraphLaunch(s->gexec, st));
-    s->launches++;
+    CK(enqueue_period(s));
     CK(cudaMemcpyAsync(&s->h_poll[nxt], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(s->ev[nxt], st));
     CK(cudaEventSynchronize(s->ev[slot]));
@@ -855,7 +885,7 @@ int pdlp_solve_warm(pdlp_solver *s, const double *x0, const double *y0, double t
 
 int pdlp_resume(pdlp_solver *s, double *x_out, double *y_out, int *status, int64_t *iters) {
   g_err.clear();
-  if (!s || !s->gexec) return fail(PDLP_ERR_INVALID, "pdlp_resume: call pdlp_begin or pdlp_set_state first");
+  if (!s || !s->ready) return fail(PDLP_ERR_INVALID, "pdlp_resume: call pdlp_begin or pdlp_set_state first");
   CK(cudaSetDevice(s->device));
   CK(cudaStreamSynchronize(s->stream));
   CK(cudaMemcpy(s->h_st, s->st, sizeof(DevState), cudaMemcpyDeviceToHost));
@@ -1155,6 +1185,7 @@ int pdlp_set_quadratic(pdlp_solver *s, const double *qdiag) {
   CK(cudaSetDevice(s->device));
   CK(cudaStreamSynchronize(s->stream));
   // the captured graph holds the kernels' arguments: rebuilt at the next begin
+  s->ready = false;
   if (s->gexec) {
     cudaGraphExecDestroy(s->gexec);
     s->gexec = nullptr;

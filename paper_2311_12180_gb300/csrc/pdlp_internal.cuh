@@ -159,8 +159,37 @@ cudaError_t launch_restart(const Vecs &V, DevState *st, int grid, cudaStream_t s
 cudaError_t launch_infeas(const Vecs &V, DevState *st, int grid, cudaStream_t s);
 cudaError_t launch_output(const Vecs &V, DevState *st, cudaStream_t s);
 cudaError_t launch_time_limit(DevState *st, cudaStream_t s);
+// ---- one check period in one launch (pdlp_period.cu) ----
+struct PeriodSync {
+  unsigned count, base;  // grid barrier: arrivals so far (only grows), their number when a launch starts
+  int error;             // 1: a barrier wait ran out
+};
+constexpr int PERIOD_CLUSTER = 16;
+constexpr int PERIOD_SHARE_MAX = 200 * 1024;
+constexpr int64_t PERIOD_WORK_MAX = 8000000;
+constexpr int PERIOD_PART_GROUPS = 4096;  // partial sums of each value: groups, or a cluster's virtual warps
+// The grids (256-thread CTAs) of the kernels whose sums a period reproduces.
+struct PeriodGrids {
+  int primal = 1, dual = 1, check_primal = 1, check_dual = 1, infeas = 1, restart = 1;
+};
+struct PeriodPlan {
+  int ctas = 0;         // 0: the LP is solved by the step and check kernels
+  bool cluster = false;
+  int share_bytes = 0;  // shared memory of a CTA's items of K and K', 0: read from the L2
+  PeriodGrids grids;
+  PeriodSync *sync = nullptr;
+  double *part = nullptr;
+};
+// decides ctas, cluster and share_bytes (p.grids set; items of K and K' in schedule order)
+void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int nk, const int4 *t_items, int nt,
+                 int64_t stored, int value_bytes, int num_sms);
+size_t period_part_doubles();
+cudaError_t period_init();
+cudaError_t launch_period(const PeriodPlan &p, const SellMat &K, const SellMat &KT, const Vecs &V, DevState *st,
+                          int max_trials, cudaStream_t s);
+
 int occupancy_grid(int kc, int num_sms);
-cudaError_t kernels_init();  // one-time kernel attributes (none needed at present)
+cudaError_t kernels_init();  // one-time kernel attributes
 
 // Records `msg` as the calling thread's pdlp_last_error() and returns `code`.
 int set_error(int code, const char *msg);
@@ -183,5 +212,24 @@ __device__ __forceinline__ double clamp_bits(double v, double l, double u) {
   return r;
 }
 
+// RN(a / b) from y = RN(1 / b) by one correction step (Markstein, IBM J. Res.
+// Dev. 34(1), 1990; Handbook of Floating-Point Arithmetic, the theorem on
+// division by an FMA correction): q = RN(a y) is within one ulp of a / b,
+// the remainder a - b q is exact with an FMA, and RN(q + (a - b q) y) is the
+// correctly rounded quotient when nothing underflows or overflows.  Where a
+// or q is outside [2^-900, 2^900] (or zero, or not finite) the plain
+// division runs instead.  Three FP64 operations instead of a division
+// routine: the Ruiz passes divide every entry twice, on GB300's narrow FP64
+// pipe.
+__device__ __forceinline__ unsigned int exp_bits(double v) {
+  return (unsigned int)((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffu;
+}
+__device__ __forceinline__ double div_rn(double a, double b, double y) {
+  const double q = a * y;
+  const unsigned int ea = exp_bits(a), eq = exp_bits(q);
+  if (ea < 1023u - 900u || ea > 1023u + 900u || eq < 1023u - 900u || eq > 1023u + 900u) return a / b;
+  const double r = fma(-b, q, a);
+  return fma(r, y, q);
+}
 
 }  // namespace pdlp

@@ -102,26 +102,6 @@ __global__ void k_recip(int32_t count, const double *D, double *rD) {
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) rD[i] = 1.0 / D[i];
 }
 
-// RN(a / b) from y = RN(1 / b) by one correction step (Markstein, IBM J. Res.
-// Dev. 34(1), 1990; Handbook of Floating-Point Arithmetic, the theorem on
-// division by an FMA correction): q = RN(a y) is within one ulp of a / b,
-// the remainder a - b q is exact with an FMA, and RN(q + (a - b q) y) is the
-// correctly rounded quotient when nothing underflows or overflows.  Where a
-// or q is outside [2^-900, 2^900] (or zero, or not finite) the plain
-// division runs instead.  Three FP64 operations instead of a division
-// routine: the Ruiz passes divide every entry twice, on GB300's narrow FP64
-// pipe.
-__device__ __forceinline__ unsigned int exp_bits(double v) {
-  return (unsigned int)((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffu;
-}
-__device__ __forceinline__ double div_rn(double a, double b, double y) {
-  const double q = a * y;
-  const unsigned int ea = exp_bits(a), eq = exp_bits(q);
-  if (ea < 1023u - 900u || ea > 1023u + 900u || eq < 1023u - 900u || eq > 1023u + 900u) return a / b;
-  const double r = fma(-b, q, a);
-  return fma(r, y, q);
-}
-
 // K's entries in storage order: val[e] = (val[e] / r[row]) / s[column], the
 // same two correctly rounded divisions in the same order as the row-wise
 // k_scale (the reciprocals rr, rs of the factors make each one three FP64
