@@ -542,8 +542,10 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
       e = setup_scale_perm(m, n, nnz, s->K_ptr, s->K_idx, s->K_val, s->T_ptr, s->T_val, rowid, perm, s->D1, s->D2,
                            s->work_m, s->work_n, VM(9), VN(12), prm.ruiz_iters, prm.pc_alpha, st);
     } else {
-      e = setup_scale(m, n, nnz, s->K_ptr, s->K_idx, s->K_val, s->T_ptr, s->T_idx, s->T_val, s->D1, s->D2,
-                      s->work_m, s->work_n, prm.ruiz_iters, prm.pc_alpha, st);
+      // norms and reciprocals in vectors that a solve writes before it reads them
+      const ScaleWork w{VM(11), VN(14), s->work_m, s->work_n, VM(9), VN(12)};
+      e = setup_scale(m, n, nnz, s->K_ptr, s->K_idx, s->K_val, s->T_ptr, s->T_idx, s->T_val, s->D1, s->D2, w,
+                      prm.ruiz_iters, prm.pc_alpha, st);
     }
     CKS(e);
     const cudaError_t ef = cudaFreeAsync(tw.p, st);

@@ -22,66 +22,163 @@ namespace {
 
 constexpr int ST = 256;
 
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 __device__ __forceinline__ double warp_add(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// One warp per row: out[r] = max_e |val[e]| (kind 0) or sum_e |val[e]|^p (kind 1).
-__global__ void k_row_norm(const int32_t *__restrict__ ptr, const double *__restrict__ val, int32_t rows,
-                           double *__restrict__ out, int kind, double p) {
+// out[r] = sum_e |val[e]|^p: lane-strided partial sums of a row over 32 lanes,
+// then the xor tree.  A row of at most G entries gives the same sum on G
+// lanes (its other partials are zeros), so a warp takes 32 rows and puts the
+// short ones on G = 1, 8 or 16 lanes: an FP64 addition costs a scheduler 64
+// cycles whatever the number of lanes.
+__global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restrict__ val, int32_t rows,
+                          double *__restrict__ out, double p) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * ST + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * ST) >> 5;
-  for (long long r = warp; r < rows; r += nwarps) {
-    const int e0 = ptr[r], e1 = ptr[r + 1];
-    double acc = 0.0;
-    for (int e = e0 + lane; e < e1; e += 32) {
-      const double a = fabs(val[e]);
-      if (kind == 0)
-        acc = fmax(acc, a);
-      else
-        acc += (p == 1.0) ? a : pow(a, p);
+  auto term = [&](int e) {
+    const double a = fabs(val[e]);
+    return (p == 1.0) ? a : pow(a, p);
+  };
+  for (long long r0 = warp * 32; r0 < rows; r0 += nwarps * 32) {
+    const bool in = r0 + lane < rows;
+    const int e0 = in ? ptr[r0 + lane] : 0, len = in ? ptr[r0 + lane + 1] - e0 : 0;
+    double sum = len == 1 ? term(e0) : 0.0;
+    unsigned left = __ballot_sync(0xffffffffu, len > 1);
+    for (int G = 8; G <= 32; G <<= 1) {  // rows of 2-8 entries, four at a time; 9-16, two; longer, one
+      unsigned todo = __ballot_sync(0xffffffffu, (left >> lane & 1u) && (len <= G || G == 32));
+      left &= ~todo;
+      while (todo) {
+        int mine = -1;  // the row (lane of it) of this lane's group
+        for (int k = 0; k < 32 / G && todo; ++k) {
+          const int l = __ffs(todo) - 1;
+          todo &= todo - 1;
+          if (lane / G == k) mine = l;
+        }
+        const int b = __shfl_sync(0xffffffffu, e0, mine & 31), n = __shfl_sync(0xffffffffu, len, mine & 31);
+        double acc = 0.0;
+        if (mine >= 0)
+          for (int e = lane % G; e < n; e += G) acc += term(b + e);
+        for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        // hand the sum to the row's lane
+        for (int k = 0; k < 32 / G; ++k) {
+          const int l = __shfl_sync(0xffffffffu, mine, k * G);
+          const double t = __shfl_sync(0xffffffffu, acc, k * G);
+          if (lane == l) sum = t;
+        }
+      }
     }
-    acc = kind == 0 ? warp_max(acc) : warp_add(acc);
-    if (lane == 0) out[r] = acc;
+    if (in) out[r0 + lane] = sum;
   }
 }
 
-// f <- sqrt(f), or 1 where the line is empty (norm 0).
-__global__ void k_factor(double *__restrict__ f, int32_t n) {
-  for (int i = blockIdx.x * ST + threadIdx.x; i < n; i += gridDim.x * ST) f[i] = f[i] > 0.0 ? sqrt(f[i]) : 1.0;
-}
-
-// K (row_is_kmajor = 1): val[e] = (val[e] / r[i]) / s[idx[e]] for row i.
-// K' (row_is_kmajor = 0): row j of K', idx = row of K: (val / r[idx]) / s[j].
-__global__ void k_scale(const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx, double *__restrict__ val,
-                        int32_t rows, const double *__restrict__ r, const double *__restrict__ s,
-                        int row_is_kmajor) {
+// Rows in storage order, SCALE_ROWS rows a warp: their entries are one
+// contiguous stream, taken 32 lanes x SCALE_U at a time whatever the rows'
+// lengths; an entry's row is found among the starts by shuffles.  SCALE: with
+// the factors r, s of K's rows and columns and their reciprocals,
+//   K  (KMAJOR):  val[e] = (val[e] / r[row]) / s[idx[e]],
+//   K' (else):    val[e] = (val[e] / r[idx[e]]) / s[row]
+// (div_rn: the correctly rounded quotients).  maxima (may be null): the row
+// maxima of |val| afterwards, as IEEE bits, by a segmented integer maximum:
+// the next Ruiz pass's norms without another pass over the matrix.
+// The FP64 pipe (6 operations an entry) and, on power-law rows, the warp with
+// the most entries bound it: the eleven passes over 3e6 nonzeros take 2.1 ms,
+// 2.7 with 32 rows a warp and one load at a time, 7.5 as warp-per-row passes
+// with plain divisions.
+constexpr int SCALE_ROWS = 8, SCALE_U = 4;
+template <bool SCALE, bool KMAJOR>
+__global__ void __launch_bounds__(ST) k_scale_rows(const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
+                                                   double *__restrict__ val, int32_t rows, const double *__restrict__ r,
+                                                   const double *__restrict__ rr, const double *__restrict__ s,
+                                                   const double *__restrict__ rs,
+                                                   unsigned long long *__restrict__ maxima) {
+  __shared__ unsigned long long smax[ST / 32][SCALE_ROWS];
   const int lane = threadIdx.x & 31;
+  unsigned long long *const mx = smax[threadIdx.x >> 5];
   const long long warp = ((long long)blockIdx.x * ST + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * ST) >> 5;
-  for (long long row = warp; row < rows; row += nwarps) {
-    const int e0 = ptr[row], e1 = ptr[row + 1];
-    for (int e = e0 + lane; e < e1; e += 32) {
-      const int o = idx[e];
-      if (row_is_kmajor)
-        val[e] = val[e] / r[row] / s[o];
-      else
-        val[e] = val[e] / r[o] / s[row];
+  for (long long r0 = warp * SCALE_ROWS; r0 < rows; r0 += nwarps * SCALE_ROWS) {
+    // starts of the warp's rows (lanes 0..SCALE_ROWS - 1) and the end of the last
+    const int start = lane <= SCALE_ROWS ? ptr[min((long long)rows, r0 + lane)] : 0;
+    const int b = __shfl_sync(0xffffffffu, start, 0), end = __shfl_sync(0xffffffffu, start, SCALE_ROWS);
+    if (lane < SCALE_ROWS) mx[lane] = 0;
+    __syncwarp();
+    for (int e0 = b; e0 < end; e0 += 32 * SCALE_U) {
+      double v[SCALE_U];
+      int o[SCALE_U], l[SCALE_U];
+#pragma unroll
+      for (int u = 0; u < SCALE_U; ++u) {
+        const int e = min(e0 + 32 * u + lane, end - 1);
+        v[u] = val[e];
+        o[u] = SCALE ? idx[e] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < SCALE_U; ++u) {
+        const int e = e0 + 32 * u + lane;
+        l[u] = 0;  // the last row that starts at or before e
+#pragma unroll
+        for (int k = SCALE_ROWS / 2; k > 0; k >>= 1)
+          if (__shfl_sync(0xffffffffu, start, l[u] + k) <= e) l[u] += k;
+      }
+      if (SCALE) {
+        double a[SCALE_U], ra[SCALE_U], c[SCALE_U], rc[SCALE_U];
+#pragma unroll
+        for (int u = 0; u < SCALE_U; ++u) {
+          const long long row = min(r0 + l[u], (long long)rows - 1), i = KMAJOR ? row : o[u], j = KMAJOR ? o[u] : row;
+          a[u] = r[i];
+          ra[u] = rr[i];
+          c[u] = s[j];
+          rc[u] = rs[j];
+        }
+#pragma unroll
+        for (int u = 0; u < SCALE_U; ++u)
+          if (e0 + 32 * u < end) {
+            v[u] = div_rn(div_rn(v[u], a[u], ra[u]), c[u], rc[u]);
+            if (e0 + 32 * u + lane < end) val[e0 + 32 * u + lane] = v[u];
+          }
+      }
+      if (maxima) {
+#pragma unroll
+        for (int u = 0; u < SCALE_U; ++u) {
+          if (e0 + 32 * u >= end) break;
+          const int key = e0 + 32 * u + lane < end ? l[u] : SCALE_ROWS;
+          unsigned long long bits = (unsigned long long)__double_as_longlong(v[u]) & 0x7fffffffffffffffull;
+#pragma unroll
+          for (int k = 1; k < 32; k <<= 1) {
+            const unsigned long long ob = __shfl_down_sync(0xffffffffu, bits, k);
+            const int ok = __shfl_down_sync(0xffffffffu, key, k);
+            if (lane + k < 32 && ok == key && ob > bits) bits = ob;
+          }
+          const int before = __shfl_up_sync(0xffffffffu, key, 1);
+          if (key < SCALE_ROWS && (lane == 0 || before != key) && bits > mx[key]) mx[key] = bits;
+          __syncwarp();
+        }
+      }
     }
+    if (maxima && lane < SCALE_ROWS && r0 + lane < rows) maxima[r0 + lane] = mx[lane];
+    __syncwarp();
   }
 }
 
-__global__ void k_div(double *__restrict__ D, const double *__restrict__ f, int32_t n) {
-  for (int i = blockIdx.x * ST + threadIdx.x; i < n; i += gridDim.x * ST) D[i] = D[i] / f[i];
+// The factors of a pass from the lines' norms, f = sqrt(norm) (1 where a line
+// is empty; may overwrite the norms), their reciprocals, and D / f, for K's
+// rows and columns at once.
+__global__ void k_factors(int32_t m, int32_t n, const double *norm_m, const double *norm_n, double *fm,
+                          double *fn, double *__restrict__ rm,
+                          double *__restrict__ rn, double *__restrict__ D1, double *__restrict__ D2) {
+  const long long total = (long long)m + n;
+  for (long long k = (long long)blockIdx.x * ST + threadIdx.x; k < total; k += (long long)gridDim.x * ST) {
+    const bool row = k < m;
+    const int i = (int)(row ? k : k - m);
+    const double a = row ? norm_m[i] : norm_n[i];
+    const double f = a > 0.0 ? sqrt(a) : 1.0;
+    double *const D = row ? D1 : D2;
+    (row ? fm : fn)[i] = f;
+    (row ? rm : rn)[i] = 1.0 / f;
+    D[i] = D[i] / f;
+  }
 }
 
 // Ruiz maxima in one pass over K's entries: the IEEE bits of |v| are
@@ -238,24 +335,30 @@ int grid_for(long long n) {
 }  // namespace
 
 cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32_t *K_idx, double *K_val,
-                        int32_t *T_ptr, int32_t *T_idx, double *T_val, double *D1, double *D2, double *work_m,
-                        double *work_n, int ruiz_iters, double pc_alpha, cudaStream_t s) {
+                        int32_t *T_ptr, int32_t *T_idx, double *T_val, double *D1, double *D2, const ScaleWork &w,
+                        int ruiz_iters, double pc_alpha, cudaStream_t s) {
   (void)nnz;
   if (m > 0) k_fill<<<grid_for(m), ST, 0, s>>>(D1, m, 1.0);
   k_fill<<<grid_for(n), ST, 0, s>>>(D2, n, 1.0);
+  unsigned long long *const mm = reinterpret_cast<unsigned long long *>(w.norm_m),
+                           *const mn = reinterpret_cast<unsigned long long *>(w.norm_n);
+  if (ruiz_iters > 0) {  // the first pass's maxima
+    if (m > 0) k_scale_rows<false, true><<<grid_for(4LL * m), ST, 0, s>>>(K_ptr, K_idx, K_val, m, nullptr, nullptr, nullptr, nullptr, mm);
+    k_scale_rows<false, false><<<grid_for(4LL * n), ST, 0, s>>>(T_ptr, T_idx, T_val, n, nullptr, nullptr, nullptr, nullptr, mn);
+  }
   const int passes = ruiz_iters + (pc_alpha >= 0.0 ? 1 : 0);
   for (int it = 0; it < passes; ++it) {
-    const bool ruiz = it < ruiz_iters;
-    const int kind = ruiz ? 0 : 1;
-    // row factors of K (one warp per row of K), column factors (rows of K')
-    if (m > 0) k_row_norm<<<grid_for((long long)m * 32), ST, 0, s>>>(K_ptr, K_val, m, work_m, kind, 2.0 - pc_alpha);
-    k_row_norm<<<grid_for((long long)n * 32), ST, 0, s>>>(T_ptr, T_val, n, work_n, kind, pc_alpha);
-    if (m > 0) k_factor<<<grid_for(m), ST, 0, s>>>(work_m, m);
-    k_factor<<<grid_for(n), ST, 0, s>>>(work_n, n);
-    if (m > 0) k_scale<<<grid_for((long long)m * 32), ST, 0, s>>>(K_ptr, K_idx, K_val, m, work_m, work_n, 1);
-    k_scale<<<grid_for((long long)n * 32), ST, 0, s>>>(T_ptr, T_idx, T_val, n, work_m, work_n, 0);
-    if (m > 0) k_div<<<grid_for(m), ST, 0, s>>>(D1, work_m, m);
-    k_div<<<grid_for(n), ST, 0, s>>>(D2, work_n, n);
+    if (it >= ruiz_iters) {  // Pock-Chambolle: row sums of K and K'
+      if (m > 0) k_row_sum<<<grid_for(m), ST, 0, s>>>(K_ptr, K_val, m, w.norm_m, 2.0 - pc_alpha);
+      k_row_sum<<<grid_for(n), ST, 0, s>>>(T_ptr, T_val, n, w.norm_n, pc_alpha);
+    }
+    k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, w.norm_m, w.norm_n, w.f_m, w.f_n, w.rcp_m, w.rcp_n, D1, D2);
+    const bool more = it + 1 < ruiz_iters;  // the next pass needs maxima
+    if (m > 0)
+      k_scale_rows<true, true><<<grid_for(4LL * m), ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+                                                          more ? mm : nullptr);
+    k_scale_rows<true, false><<<grid_for(4LL * n), ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+                                                         more ? mn : nullptr);
   }
   return cudaGetLastError();
 }
@@ -274,25 +377,15 @@ cudaError_t setup_scale_perm(int32_t m, int32_t n, int64_t nnz, const int32_t *K
     if (nnz > 0)
       k_entry_max<<<eg, ST, 0, s>>>(K_idx, rowid, K_val, nnz, reinterpret_cast<unsigned long long *>(work_m),
                                     reinterpret_cast<unsigned long long *>(work_n));
-    if (m > 0) k_factor<<<grid_for(m), ST, 0, s>>>(work_m, m);
-    k_factor<<<grid_for(n), ST, 0, s>>>(work_n, n);
-    if (m > 0) k_recip<<<grid_for(m), ST, 0, s>>>(m, work_m, rcp_m);
-    k_recip<<<grid_for(n), ST, 0, s>>>(n, work_n, rcp_n);
+    k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, work_m, work_n, work_m, work_n, rcp_m, rcp_n, D1, D2);
     if (nnz > 0) k_scale_entries<<<eg, ST, 0, s>>>(K_idx, rowid, K_val, nnz, work_m, work_n, rcp_m, rcp_n);
-    if (m > 0) k_div<<<grid_for(m), ST, 0, s>>>(D1, work_m, m);
-    k_div<<<grid_for(n), ST, 0, s>>>(D2, work_n, n);
   }
   if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);
   if (pc_alpha >= 0.0) {  // Pock-Chambolle: row sums over K, column sums over K' (fixed order)
-    if (m > 0) k_row_norm<<<grid_for((long long)m * 32), ST, 0, s>>>(K_ptr, K_val, m, work_m, 1, 2.0 - pc_alpha);
-    k_row_norm<<<grid_for((long long)n * 32), ST, 0, s>>>(T_ptr, T_val, n, work_n, 1, pc_alpha);
-    if (m > 0) k_factor<<<grid_for(m), ST, 0, s>>>(work_m, m);
-    k_factor<<<grid_for(n), ST, 0, s>>>(work_n, n);
-    if (m > 0) k_recip<<<grid_for(m), ST, 0, s>>>(m, work_m, rcp_m);
-    k_recip<<<grid_for(n), ST, 0, s>>>(n, work_n, rcp_n);
+    if (m > 0) k_row_sum<<<grid_for(m), ST, 0, s>>>(K_ptr, K_val, m, work_m, 2.0 - pc_alpha);
+    k_row_sum<<<grid_for(n), ST, 0, s>>>(T_ptr, T_val, n, work_n, pc_alpha);
+    k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, work_m, work_n, work_m, work_n, rcp_m, rcp_n, D1, D2);
     if (nnz > 0) k_scale_entries<<<eg, ST, 0, s>>>(K_idx, rowid, K_val, nnz, work_m, work_n, rcp_m, rcp_n);
-    if (m > 0) k_div<<<grid_for(m), ST, 0, s>>>(D1, work_m, m);
-    k_div<<<grid_for(n), ST, 0, s>>>(D2, work_n, n);
     if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);
   }
   return cudaGetLastError();
@@ -754,8 +847,8 @@ cudaError_t setup_permute(int32_t count, const int32_t *perm, const double *src,
 // ---------------------------------------------------------------------------
 // Allocation-free variant of the scaling pass (pdlp_scale_device_noalloc).
 //
-// The per-pass row and column factors of setup_scale live in this file-scope
-// device array instead of in memory the solver allocates.  The array's host
+// The per-pass row and column norms, factors and reciprocals of setup_scale
+// live in this file-scope device array instead of in memory the solver allocates.  The array's host
 // symbol is only a host-side stand-in: kernels receive the device address
 // looked up once per device with cudaGetSymbolAddress (under a lock, with
 // that device current) on the first call made on the device.
@@ -763,7 +856,7 @@ cudaError_t setup_permute(int32_t count, const int32_t *perm, const double *src,
 namespace {
 
 constexpr int32_t NOALLOC_MAX_LINES = 1 << 18;  // rows and columns, each
-__device__ __align__(256) double g_scale_scratch[2 * NOALLOC_MAX_LINES];
+__device__ __align__(256) double g_scale_scratch[6 * NOALLOC_MAX_LINES];
 
 constexpr int MAX_DEVICES = 256;
 std::mutex g_scratch_mu;
@@ -802,9 +895,11 @@ extern "C" int pdlp_scale_device_noalloc(int32_t m, int32_t n, const int32_t *K_
     }
     scratch = g_scratch_dev[dev];
   }
-  double *work_m = scratch, *work_n = scratch + NOALLOC_MAX_LINES;
+  double *const p = scratch;
+  const ScaleWork w{p, p + NOALLOC_MAX_LINES, p + 2 * NOALLOC_MAX_LINES, p + 3 * NOALLOC_MAX_LINES,
+                    p + 4 * NOALLOC_MAX_LINES, p + 5 * NOALLOC_MAX_LINES};
   e = setup_scale(m, n, 0, const_cast<int32_t *>(K_ptr), const_cast<int32_t *>(K_idx), K_val,
-                  const_cast<int32_t *>(KT_ptr), const_cast<int32_t *>(KT_idx), KT_val, D1, D2, work_m, work_n,
+                  const_cast<int32_t *>(KT_ptr), const_cast<int32_t *>(KT_idx), KT_val, D1, D2, w,
                   ruiz_iters, pc_alpha, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return set_error(PDLP_ERR_CUDA, cudaGetErrorString(e));
   return PDLP_OK;
