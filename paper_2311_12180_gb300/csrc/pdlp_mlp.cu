@@ -132,8 +132,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 // described by the tensor maps (box TBK x 128, 128-byte swizzle).  Thread 0
 // issues the TMA loads and the MMAs; the finished tile passes through
 // epi.chunk(m, n, values, count, split) -- 16 consecutive columns n.. of
-// row m, count of them inside the matrix -- for m < M, then epi.finish()
-// runs in every thread.  A wait that exceeds its limit sets *err and skips the epilogue.
+// row m, count of them inside the matrix -- for m < M (epi.prefetch(m, n, N)
+// before the first), then epi.finish() runs in every thread.  A wait that exceeds its limit sets *err and skips the epilogue.
 template <class Epi>
 __global__ void __launch_bounds__(GEMM_THREADS) k_tc_gemm(const __grid_constant__ CUtensorMap ma,
                                                  const __grid_constant__ CUtensorMap mb, int M, int N, int K,
@@ -203,13 +203,15 @@ __global__ void __launch_bounds__(GEMM_THREADS) k_tc_gemm(const __grid_constant_
     }
     umma_commit(done);  // arrives when every MMA issued above has completed
   }
+  // the epilogue's first operands are on their way while the MMAs finish
+  const int quarter = warp & 3, half = warp >> 2;
+  const int row = m0 + quarter * 32 + lane;
+  if (row < M && n0 + half * (TBN / 2) < N) epi.prefetch(row, n0 + half * (TBN / 2), N);
   __syncthreads();
   const bool ok = mbar_wait(done, 0);
   if (!ok) atomicExch(err, GEMM_ERR_DONE);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   // a split with an empty K range never wrote its accumulator: its tile is zero
-  const int quarter = warp & 3, half = warp >> 2;
-  const int row = m0 + quarter * 32 + lane;
 #pragma unroll 1
   for (int c0 = half * (TBN / 2); c0 < (half + 1) * (TBN / 2) && ok; c0 += 16) {
     float v[16];
@@ -257,6 +259,7 @@ __device__ __forceinline__ void st16_bf16(bf16 *p, const bf16 (&h)[16]) {
 }
 
 struct EpiBase {
+  __device__ __forceinline__ void prefetch(int, int, int) {}
   __device__ __forceinline__ void finish() {}
 };
 // hidden layer: H = bf16(relu(z + b)), stored as H (rows x hidden, ld a
@@ -311,15 +314,23 @@ struct EpiLoss {
   int ldt, ldh, ldT;
   bool vec;  // t / dy rows allow 16-byte accesses
   double acc;
-  __device__ __forceinline__ void chunk(int m, int n, const float (&v)[16], int cnt, int) {
-    float tv[16];
+  int ncols;
+  float tn[16];  // targets of the next chunk: a chunk's loads take as long as its arithmetic
+  __device__ __forceinline__ void prefetch(int m, int n, int N) {
+    ncols = N;
     const float *tr = t + (size_t)rows[m] * ldt;
-    if (vec && cnt == 16) {
-      ld16_f32(tr + n, tv);
+    if (vec && n + 16 <= N) {
+      ld16_f32(tr + n, tn);
     } else {
 #pragma unroll
-      for (int j = 0; j < 16; ++j) tv[j] = j < cnt ? tr[n + j] : 0.0f;
+      for (int j = 0; j < 16; ++j) tn[j] = n + j < N ? tr[n + j] : 0.0f;
     }
+  }
+  __device__ __forceinline__ void chunk(int m, int n, const float (&v)[16], int cnt, int) {
+    float tv[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tv[j] = tn[j];
+    if ((n + 16) % (TBN / 2) != 0 && n + 16 < ncols) prefetch(m, n + 16, ncols);
     float g[16];
     __align__(16) bf16 gh[16];
     float sq = 0.0f;
@@ -508,18 +519,70 @@ __global__ void k_unstandardize(const float *__restrict__ y, size_t count, int o
   }
 }
 
-// Adam on the FP32 master copy.
-__global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m1,
-                       float *__restrict__ m2, size_t count, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float a = b1 * m1[i] + (1.0f - b1) * gi;
-    const float b = b2 * m2[i] + (1.0f - b2) * gi * gi;
-    m1[i] = a;
-    m2[i] = b;
-    const float mh = a / c1, vh = b / c2;
-    p[i] = p[i] - lr * mh / (sqrtf(vh) + eps);
+// Adam on the FP32 master copy and the BF16 copies of the updated weights, in
+// one pass: a block takes a 32 x 32 tile of a weight matrix (W as rows x cols
+// with ld ldw, skipped when wb is null, and W' with ld ldt through shared
+// memory, so that every access is coalesced) or 1024 bias entries.  Bound by
+// HBM: 28 bytes of FP32 state and 4 of BF16 per weight.  On the 16-256-256-
+// 60500 network Adam and the three conversions after it took 134 us of a 0.51
+// ms step in four launches, the weights read once more in between; with this
+// (and the loss's targets loaded a chunk ahead) the step takes 0.47 ms.
+struct AdamTiles {
+  size_t off;  // of the block in the flat parameters
+  int rows, cols, tiles;
+  bf16 *wb, *wt;  // null wt: a bias
+  int ldw, ldt;
+};
+struct AdamPlan {
+  AdamTiles part[6];
+};
+struct AdamRule {
+  float lr, b1, b2, eps, c1, c2;
+};
+__device__ __forceinline__ float adam_update(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m1,
+                                             float *__restrict__ m2, size_t i, const AdamRule &r) {
+  const float gi = g[i];
+  const float a = r.b1 * m1[i] + (1.0f - r.b1) * gi;
+  const float b = r.b2 * m2[i] + (1.0f - r.b2) * gi * gi;
+  m1[i] = a;
+  m2[i] = b;
+  const float mh = a / r.c1, vh = b / r.c2;
+  const float v = p[i] - r.lr * mh / (sqrtf(vh) + r.eps);
+  p[i] = v;
+  return v;
+}
+__global__ void __launch_bounds__(256) k_adam(float *__restrict__ p, const float *__restrict__ g,
+                                              float *__restrict__ m1, float *__restrict__ m2, const AdamPlan plan,
+                                              AdamRule rule) {
+  __shared__ float tile[32][33];
+  int t = blockIdx.x, k = 0;
+#pragma unroll
+  for (; k < 5; ++k) {
+    if (t < plan.part[k].tiles) break;
+    t -= plan.part[k].tiles;
+  }
+  const AdamTiles a = plan.part[k];
+  if (!a.wt) {
+    for (int i = t * 1024 + threadIdx.x; i < min(a.cols, (t + 1) * 1024); i += 256)
+      adam_update(p, g, m1, m2, a.off + i, rule);
+    return;
+  }
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
+  const int across = (a.cols + 31) / 32, c0 = (t % across) * 32, r0 = (t / across) * 32;
+#pragma unroll
+  for (int q = ty; q < 32; q += 8) {
+    const int r = r0 + q, c = c0 + tx;
+    if (r < a.rows && c < a.cols) {
+      const float v = adam_update(p, g, m1, m2, a.off + (size_t)r * a.cols + c, rule);
+      tile[q][tx] = v;
+      if (a.wb) a.wb[(size_t)r * a.ldw + c] = __float2bfloat16(v);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = ty; q < 32; q += 8) {
+    const int c = c0 + q, r = r0 + tx;
+    if (r < a.rows && c < a.cols) a.wt[(size_t)c * a.ldt + r] = __float2bfloat16(tile[tx][q]);
   }
 }
 
@@ -693,6 +756,23 @@ int refresh_weights(pdlp_mlp *M) {
   return PDLP_OK;
 }
 
+// One Adam step from M->g, the BF16 copies included.
+int adam_step(pdlp_mlp *M, const AdamRule &rule) {
+  auto mat = [](size_t off, int rows, int cols, bf16 *wb, int ldw, bf16 *wt, int ldt) {
+    return AdamTiles{off, rows, cols, ((rows + 31) / 32) * ((cols + 31) / 32), wb, wt, ldw, ldt};
+  };
+  auto vec = [](size_t off, int count) { return AdamTiles{off, 1, count, (count + 1023) / 1024, nullptr, nullptr, 0, 0}; };
+  const AdamPlan plan{{mat(M->oW3, M->hid, M->out, M->w3, M->ldo, M->w3t, M->ldh),
+                       mat(M->oW2, M->hid, M->hid, M->w2, M->ldh, M->w2t, M->ldh),
+                       mat(M->oW1, M->in, M->hid, nullptr, 0, M->w1t, M->ldi), vec(M->ob3, M->out),
+                       vec(M->ob2, M->hid), vec(M->ob1, M->hid)}};
+  long long blocks = 0;
+  for (const AdamTiles &a : plan.part) blocks += a.tiles;
+  k_adam<<<(unsigned)blocks, 256, 0, M->stream>>>(M->p, M->g, M->m1, M->m2, plan, rule);
+  MCK(cudaGetLastError());
+  return PDLP_OK;
+}
+
 // hidden layers for rows [0, B) of xb
 int forward_hidden(pdlp_mlp *M, int B) {
   int rc = gemm(M, B, M->hid, M->in, 1, M->xb, M->ldi, M->w1t, M->ldi,
@@ -703,19 +783,19 @@ int forward_hidden(pdlp_mlp *M, int B) {
   return rc;
 }
 
-// loss (fused into the output layer) and every gradient into M->g for the
-// batch in xb / tb
-int forward_backward(pdlp_mlp *M, int B, const int *rows) {
+// loss (fused into the output layer, to *loss on the device) and every
+// gradient into M->g for the batch in xb / tb
+int forward_backward(pdlp_mlp *M, int B, const int *rows, float *loss) {
   cudaStream_t s = M->stream;
   int rc = forward_hidden(M, B);
   if (rc) return rc;
   const size_t BO = (size_t)B * M->out, BH = (size_t)B * M->hid;
   const int tiles = ((M->out + TBN - 1) / TBN) * ((B + TBM - 1) / TBM);
   EpiLoss el{M->p + M->ob3, M->T, M->mu, M->sigma, rows, M->dy, M->dyh, M->dyhT, M->lpart, 2.0f / (float)BO,
-             M->out, M->ldo, M->ldb, vec4(M->T, M->out) && vec4(M->dy, M->out), 0.0};
+             M->out, M->ldo, M->ldb, vec4(M->T, M->out) && vec4(M->dy, M->out), 0.0, 0, {}};
   rc = gemm(M, B, M->out, M->hid, 1, M->h2, M->ldh, M->w3t, M->ldh, el);
   if (rc) return rc;
-  k_loss_finish<<<1, 256, 0, s>>>(M->lpart, tiles, BO, M->loss_dev);
+  k_loss_finish<<<1, 256, 0, s>>>(M->lpart, tiles, BO, loss);
   // output layer: gW3 = H2' dY, gb3 = column sums of dY, dH2 = dY W3'
   rc = gemm(M, M->hid, M->out, B, 1, M->h2T, M->ldb, M->dyhT, M->ldb, EpiStore{{}, M->g + M->oW3, M->out, vec4(M->g + M->oW3, M->out)});
   if (rc) return rc;
@@ -937,14 +1017,11 @@ int pdlp_mlp_train(pdlp_mlp *M, int32_t steps, int32_t batch, const int32_t *idx
     const int *rows = M->idx + (size_t)st * batch;
     k_gather<<<batch, 64, 0, s>>>(M->X, rows, batch, M->in, M->xb, M->ldi, M->xbT, M->ldb);
     MCK(cudaGetLastError());
-    rc = forward_backward(M, batch, rows);
+    rc = forward_backward(M, batch, rows, dloss + st);
     if (rc) return rc;
-    MCK(cudaMemcpyAsync(dloss + st, M->loss_dev, sizeof(float), cudaMemcpyDeviceToDevice, s));
     ++M->adam_t;
     const float c1 = 1.0f - powf(beta1, (float)M->adam_t), c2 = 1.0f - powf(beta2, (float)M->adam_t);
-    k_adam<<<grid1(M->nparam), 256, 0, s>>>(M->p, M->g, M->m1, M->m2, M->nparam, lr, beta1, beta2, eps, c1, c2);
-    MCK(cudaGetLastError());
-    rc = refresh_weights(M);
+    rc = adam_step(M, AdamRule{lr, beta1, beta2, eps, c1, c2});
     if (rc) return rc;
   }
   if (losses) MCK(cudaMemcpyAsync(losses, dloss, sizeof(float) * steps, cudaMemcpyDeviceToHost, s));
@@ -992,7 +1069,7 @@ int pdlp_mlp_gradients(pdlp_mlp *M, int32_t batch, const int32_t *idx, float *lo
   cudaStream_t s = M->stream;
   MCK(cudaMemcpyAsync(M->idx, idx, sizeof(int) * batch, cudaMemcpyHostToDevice, s));
   k_gather<<<batch, 64, 0, s>>>(M->X, M->idx, batch, M->in, M->xb, M->ldi, M->xbT, M->ldb);
-  rc = forward_backward(M, batch, M->idx);
+  rc = forward_backward(M, batch, M->idx, M->loss_dev);
   if (rc) return rc;
   if (loss) MCK(cudaMemcpyAsync(loss, M->loss_dev, sizeof(float), cudaMemcpyDeviceToHost, s));
   if (grads) MCK(cudaMemcpyAsync(grads, M->g, sizeof(float) * M->nparam, cudaMemcpyDeviceToHost, s));
