@@ -27,6 +27,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <numeric>
 #include <string>
 #include <vector>
@@ -113,31 +114,44 @@ __device__ __forceinline__ double wmax(double v) {
   return v;
 }
 
-// CTA-wide sums of NV values, result in every thread (fixed order).  A warp
-// whose values are all zero (no rows of a small LP) skips its FP64 shuffle
-// tree: GB300 issues FP64 at a small fraction of the FP32 rate, so the trees
-// of idle warps would dominate a small LP's iteration.
+// Warp sums of NV values, written per warp to red[a * NWB + warp]; ends with a
+// CTA barrier.  A warp whose values are all zero (no rows of a small LP) skips
+// its FP64 shuffle tree, and the trees are one transposed butterfly: an FP64
+// warp instruction costs a scheduler 64 cycles, so three values' plain trees
+// (15 additions a warp, 6 here) would take a third of a small LP's iteration.
 template <int NV>
-__device__ __forceinline__ void allsum(double (&v)[NV], double *red) {
+__device__ __forceinline__ void warp_partials(double (&v)[NV], double *red) {
+  constexpr int NP = pow2_at_least(NV), SPAN = 32 / NP;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   bool any = false;
 #pragma unroll
   for (int a = 0; a < NV; ++a) any |= __double_as_longlong(v[a]) != 0;
-  if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) v[a] = wsum(v[a]);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) red[a * NWB + wid] = v[a];
-  }
+  if (__any_sync(0xffffffffu, any)) butterfly<NV, NP, 16>(v, lane);
+  if (lane % SPAN == 0 && lane / SPAN < NV) red[(lane / SPAN) * NWB + wid] = v[0];
   __syncthreads();
-  if (wid == 0) {
+}
+
+// The CTA's sums of values a0..a0 + 3 from the warps' partials, by one warp:
+// eight lanes a value, value a0 + k in lanes 8 k.. (the xor tree over 16).
+template <int NV>
+__device__ __forceinline__ double warps_sum4(const double *red, int a0) {
+  static_assert(NWB == 16, "two partials a lane");
+  const int lane = threadIdx.x & 31, a = a0 + (lane >> 3), l = lane & 7;
+  double s = a < NV ? red[a * NWB + l] + red[a * NWB + l + 8] : 0.0;
 #pragma unroll
-    for (int a = 0; a < NV; ++a) {
-      const double s = wsum(lane < NWB ? red[a * NWB + lane] : 0.0);
-      if (lane == 0) red[16 * NWB + a] = s;
-    }
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// CTA-wide sums of NV values, result in every thread (fixed order).
+template <int NV>
+__device__ __forceinline__ void allsum(double (&v)[NV], double *red) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  warp_partials<NV>(v, red);
+  if (wid < (NV + 3) / 4) {
+    const double s = warps_sum4<NV>(red, 4 * wid);
+    const int a = 4 * wid + (lane >> 3);
+    if ((lane & 7) == 0 && a < NV) red[16 * NWB + a] = s;
   }
   __syncthreads();
 #pragma unroll
@@ -158,26 +172,6 @@ __device__ __forceinline__ double allmax(double v, double *red) {
   v = red[16 * NWB];
   __syncthreads();
   return v;
-}
-
-// Warp sums of NV values (warps whose values are all zero skip the FP64
-// shuffle tree, as in allsum), written per warp to red[a * NWB + warp];
-// ends with a CTA barrier.
-template <int NV>
-__device__ __forceinline__ void warp_partials(double (&v)[NV], double *red) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  bool any = false;
-#pragma unroll
-  for (int a = 0; a < NV; ++a) any |= __double_as_longlong(v[a]) != 0;
-  if (__any_sync(0xffffffffu, any)) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) v[a] = wsum(v[a]);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) red[a * NWB + wid] = v[a];
-  }
-  __syncthreads();
 }
 
 // Loads of vectors that the solve itself writes.  A team of CTAs (below)
@@ -202,6 +196,8 @@ struct Solo {
   static constexpr bool kTeam = false;
   __device__ __forceinline__ int rank() const { return 0; }
   __device__ __forceinline__ int size() const { return 1; }
+  __device__ __forceinline__ int first() const { return threadIdx.x; }
+  __device__ __forceinline__ int step() const { return NTB; }
   __device__ __forceinline__ bool sync() {
     __syncthreads();
     return true;
@@ -216,12 +212,14 @@ struct Solo {
   // barriers instead of allsum's three plus one for the broadcast.
   template <int NV, class F>
   __device__ __forceinline__ bool reduce_apply(double (&v)[NV], double *red, F &&f) {
+    static_assert(NV <= 4, "one warp adds the warps' partials");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     warp_partials<NV>(v, red);
     if (wid == 0) {
+      const double s = warps_sum4<NV>(red, 0);
       double t[NV];
 #pragma unroll
-      for (int a = 0; a < NV; ++a) t[a] = wsum(lane < NWB ? red[a * NWB + lane] : 0.0);
+      for (int a = 0; a < NV; ++a) t[a] = __shfl_sync(0xffffffffu, s, 8 * a);
       if (lane == 0) f(t);
     }
     __syncthreads();
@@ -233,11 +231,12 @@ struct Solo {
 struct TeamState {
   unsigned *cnt, *gen;  // barrier arrival counter and generation
   int *q;               // queue position broadcast by the team leader
-  double *slots;        // [team][2][TEAM][16] partial sums
+  double *slots;        // [team][2][TEAM_SLOTS] partial sums
   int *abort;           // set when a barrier wait times out
-  int teams;
+  int teams, size;      // CTAs per team: RANKS, 2 RANKS or 4 RANKS
 };
-constexpr int TEAM = 4;                 // CTAs per team
+constexpr int RANKS = 4;                     // virtual ranks of a team: its sums' order (see Team)
+constexpr int TEAM_SLOTS = RANKS * 16 * NWB;  // 16 values of every virtual warp
 constexpr int BACK_CTAS = 16;           // CTAs that start from the small end of the queue
 constexpr long long TEAM_MIN_NNZ = 32768;  // LPs at least this large are solved by a team
 // lanes-per-row rule of an LP solved by one CTA: SOLO_FILL = false: the
@@ -249,21 +248,35 @@ constexpr double SOLO_TARGET = 4.0;
 constexpr bool SOLO_FILL = false;
 constexpr unsigned long long TEAM_WAIT_NS = 2000000000ull;
 
-// An LP solved by TEAM CTAs (one per SM): rows and vector entries are dealt
-// round-robin in chunks, partial sums meet in global slots read in rank order
-// (every CTA obtains bitwise the same sums and therefore takes the same
-// decisions), and phases are separated by a sense-reversing barrier on a
-// global counter whose spin is bounded: a wait longer than TEAM_WAIT_NS sets
-// the abort flag, and every CTA of the batch then leaves its loops.
+// An LP solved by a team of CTAs (one per SM).  Rows are dealt round-robin in
+// chunks over all of them.  Sums over vector entries keep one order whatever
+// the team's size: the entries belong to RANKS virtual CTAs of NTB threads,
+// each of which is run, some of its warps each, by size / RANKS of the team's
+// CTAs; the warps' partial sums meet in global slots, and every CTA adds a
+// virtual CTA's warps (the tree of allsum) and the virtual CTAs in rank order,
+// so that all obtain bitwise the same sums, take the same decisions, and an
+// LP's results do not depend on the size.  Phases are separated by a
+// sense-reversing barrier on a global counter whose spin is bounded: a wait
+// longer than TEAM_WAIT_NS sets the abort flag, and every CTA of the batch
+// then leaves its loops.
 struct Team {
   static constexpr bool kTeam = true;
-  int r;
+  int r, n;  // this CTA's place in the team, the team's size
   unsigned *cnt, *gen;
   double *slots;
   int *abort;
   int buf;
   __device__ __forceinline__ int rank() const { return r; }
-  __device__ __forceinline__ int size() const { return TEAM; }
+  __device__ __forceinline__ int size() const { return n; }
+  // this thread's first entry, and the step: virtual thread vthread() of RANKS x NTB
+  __device__ __forceinline__ int warps() const { return NWB * RANKS / n; }  // virtual warps of a CTA
+  __device__ __forceinline__ int vrank() const { return r * RANKS / n; }
+  __device__ __forceinline__ int vwarp() const { return (r % (n / RANKS)) * warps() + (int)(threadIdx.x >> 5); }
+  __device__ __forceinline__ bool active() const { return (int)(threadIdx.x >> 5) < warps(); }
+  __device__ __forceinline__ int first() const {
+    return active() ? vrank() * NTB + 32 * vwarp() + (int)(threadIdx.x & 31) : 0x7fffffff;
+  }
+  __device__ __forceinline__ int step() const { return RANKS * NTB; }
   __device__ bool sync() {
     __shared__ int s_ok;
     __syncthreads();
@@ -276,7 +289,7 @@ struct Team {
       // everything the earlier arrivals released and passes it on through the
       // generation, which the waiting CTAs acquire
       asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(cnt) : "memory");
-      if (old == TEAM - 1) {
+      if (old == (unsigned)n - 1) {
         asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(cnt) : "memory");
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gen) : "memory");
       } else {
@@ -297,58 +310,61 @@ struct Team {
     __syncthreads();
     return s_ok != 0;
   }
+  // The team's sums of NV values, value a in red[RED_TEAM + a] of every CTA
+  // (behind a CTA barrier).
   template <int NV>
-  __device__ bool reduce(double (&v)[NV], double *red) {
-    static_assert(NV <= 16, "16 slots per rank");
-    allsum<NV>(v, red);
-    double *sl = slots + (size_t)buf * TEAM * 16;
-    if (threadIdx.x == 0) {
+  __device__ __forceinline__ bool team_sums(double (&v)[NV], double *red) {
+    static_assert(NV <= 16 && NV * RANKS <= 4 * NWB, "slots, and four sums a warp");
+    constexpr int NP = pow2_at_least(NV), SPAN = 32 / NP;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double *sl = slots + (size_t)buf * TEAM_SLOTS;
+    buf ^= 1;  // a rank rewrites this buffer only after the next barrier
+    if (active()) {
+      bool any = false;
 #pragma unroll
-      for (int a = 0; a < NV; ++a) sl[r * 16 + a] = v[a];
+      for (int a = 0; a < NV; ++a) any |= __double_as_longlong(v[a]) != 0;
+      if (__any_sync(0xffffffffu, any)) butterfly<NV, NP, 16>(v, lane);
+      if (lane % SPAN == 0 && lane / SPAN < NV) sl[(vrank() * NV + lane / SPAN) * NWB + vwarp()] = v[0];
     }
     const bool ok = sync();
-    if (threadIdx.x == 0) {
+    if (wid < (NV * RANKS + 3) / 4) {  // eight lanes a (rank, value): the tree over its sixteen warps
+      const int t = 4 * wid + (lane >> 3), l = lane & 7;
+      double s = t < NV * RANKS ? __ldcg(sl + t * NWB + l) + __ldcg(sl + t * NWB + l + 8) : 0.0;
 #pragma unroll
-      for (int a = 0; a < NV; ++a) {
-        double t = 0.0;
-        for (int k = 0; k < TEAM; ++k) t += __ldcg(sl + k * 16 + a);
-        red[RED_TEAM + a] = t;
-      }
+      for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (l == 0 && t < NV * RANKS) red[t] = s;
     }
+    __syncthreads();
+    if (threadIdx.x < NV) {  // the ranks in order
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < RANKS; ++k) s += red[k * NV + threadIdx.x];
+      red[RED_TEAM + threadIdx.x] = s;
+    }
+    return ok;
+  }
+  template <int NV>
+  __device__ bool reduce(double (&v)[NV], double *red) {
+    const bool ok = team_sums<NV>(v, red);
     __syncthreads();
 #pragma unroll
     for (int a = 0; a < NV; ++a) v[a] = red[RED_TEAM + a];
     __syncthreads();
-    buf ^= 1;  // the other buffer: a rank rewrites this one only after the next barrier
     return ok;
   }
   // As Solo::reduce_apply over the whole team: every CTA's thread 0 gets the
-  // same team sums (rank order) and runs f.
+  // same team sums and runs f.
   template <int NV, class F>
   __device__ bool reduce_apply(double (&v)[NV], double *red, F &&f) {
-    static_assert(NV <= 16, "16 slots per rank");
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    warp_partials<NV>(v, red);
-    double *sl = slots + (size_t)buf * TEAM * 16;
-    if (wid == 0) {
-#pragma unroll
-      for (int a = 0; a < NV; ++a) {
-        const double c = wsum(lane < NWB ? red[a * NWB + lane] : 0.0);
-        if (lane == 0) sl[r * 16 + a] = c;
-      }
-    }
-    const bool ok = sync();
+    const bool ok = team_sums<NV>(v, red);
+    __syncwarp();
     if (threadIdx.x == 0) {
       double t[NV];
 #pragma unroll
-      for (int a = 0; a < NV; ++a) {
-        t[a] = 0.0;
-        for (int k = 0; k < TEAM; ++k) t[a] += __ldcg(sl + k * 16 + a);
-      }
+      for (int a = 0; a < NV; ++a) t[a] = red[RED_TEAM + a];
       f(t);
     }
     __syncthreads();
-    buf ^= 1;
     return ok;
   }
 };
@@ -717,7 +733,7 @@ __device__ void solve_instance(const Arrays &A, const Inst &I, const Params &p, 
   constexpr bool CG = Grp::kTeam;
   const int m = I.m, n = I.n, tid = threadIdx.x;
   // this CTA's share of the element loops and of the row loops
-  const int part = grp.rank(), parts = grp.size(), e0 = part * NTB + tid, es = parts * NTB;
+  const int part = grp.rank(), parts = grp.size(), e0 = grp.first(), es = grp.step();
   const int *kp = A.kptr + I.kp, *ki = A.kidx + I.ke, *tp = A.tptr + I.tp, *ti = A.tidx + I.te;
   const double *kv = A.kval + I.ke, *tv = A.tval + I.te;
   double *vm = A.vm + I.om, *vn = A.vn + I.on;
@@ -746,6 +762,7 @@ __device__ void solve_instance(const Arrays &A, const Inst &I, const Params &p, 
   bool ok = grp.sync();
   double eta = I.eta0, omega = I.omega0, W = 0.0, kkt_start, kkt_prev;
   double tau = eta / omega, sigma = eta * omega;  // primal / dual step sizes
+  double romega = 1.0 / omega;  // quotients by omega: one correction step (div_rn) instead of a division
   long long k = 0, t = 0;
   int cur = 0, need_g = 0, status = ST_RUNNING, which = 0;
   // KKT(z^{0,0}) with omega^0
@@ -818,14 +835,14 @@ __device__ void solve_instance(const Arrays &A, const Inst &I, const Params &p, 
     // LP on GB300's narrow FP64 pipe
     auto step = [&](const double (&q3)[3]) {
       const double ia = fabs(q3[2]);
-      const double eb = ia > 0.0 ? (omega * q3[0] + q3[1] / omega) / (2.0 * ia) : CUDART_INF;
+      const double eb = ia > 0.0 ? fma(omega, q3[0], div_rn(q3[1], omega, romega)) / (2.0 * ia) : CUDART_INF;
       const double kk = (double)(k + 2);
       const double p3 = k < p.npw ? p.pw[k] : pow(kk, -0.3), p6 = k < p.npw ? p.pw[p.npw + k] : pow(kk, -0.6);
       const double e1 = (1.0 - p3) * eb, e2 = (1.0 + p6) * eta;
       const double en = e1 < e2 ? e1 : e2;
       const bool accept = eta <= eb;
       red[RED_BCAST] = en;
-      red[RED_BCAST + 1] = en / omega;
+      red[RED_BCAST + 1] = div_rn(en, omega, romega);
       red[RED_BCAST + 2] = en * omega;
       red[RED_BCAST + 3] =
           (!isfinite(q3[0]) || !isfinite(q3[1]) || !isfinite(q3[2]) || isnan(eb) || !(en > 0.0)) ? 1.0 : 0.0;
@@ -1001,9 +1018,11 @@ __device__ void solve_instance(const Arrays &A, const Inst &I, const Params &p, 
       red[RED_BCAST + 4] = cand_avg ? kkt_omega(s[11], s[4], pa, da, om) : kkt_omega(s[8], s[0], pc, dc, om);
       red[RED_BCAST + 5] = eta / om;
       red[RED_BCAST + 6] = eta * om;
+      red[RED_BCAST + 7] = 1.0 / om;
     }
     __syncthreads();
     omega = red[RED_BCAST + 3];
+    romega = red[RED_BCAST + 7];
     kkt_start = red[RED_BCAST + 4];
     kkt_prev = kkt_start;
     tau = red[RED_BCAST + 5];
@@ -1135,9 +1154,9 @@ __device__ __forceinline__ int claim_back(const Arrays &A, const Inst *__restric
 }
 
 // Persistent solver over the queue `order` (largest LPs first).  The first
-// ts.teams * TEAM CTAs work in teams of TEAM (CTA b in team b / TEAM) from
+// ts.teams * ts.size CTAs work in teams (CTA b in team b / ts.size) from
 // the front: the team leader claims the next LP and, while it has at least
-// TEAM_MIN_NNZ nonzeros, all TEAM CTAs solve it together, so one large LP
+// TEAM_MIN_NNZ nonzeros, all its CTAs solve it together, so one large LP
 // that needs many iterations no longer holds a single SM for the whole
 // batch; from the first smaller LP on, the team disbands and each of its
 // CTAs claims LPs alone.  The remaining CTAs start alone from the back, on
@@ -1150,11 +1169,11 @@ __global__ void __launch_bounds__(NTB) k_batch_solve(Arrays A, const Inst *__res
   __shared__ double red[RED_SIZE];
   __shared__ int s_id;
   extern __shared__ __align__(16) unsigned char bsm[];
-  const int team = blockIdx.x / TEAM;
+  const int team = blockIdx.x / ts.size;
   if (team < ts.teams) {
     if (p.stall && blockIdx.x == 1) return;
-    Team grp{(int)(blockIdx.x % TEAM), ts.cnt + team, ts.gen + team, ts.slots + (size_t)team * 2 * TEAM * 16,
-             ts.abort, 0};
+    Team grp{(int)(blockIdx.x % ts.size), ts.size, ts.cnt + team, ts.gen + team,
+             ts.slots + (size_t)team * 2 * TEAM_SLOTS, ts.abort, 0};
     for (;;) {
       if (grp.rank() == 0 && threadIdx.x == 0) ts.q[team] = claim_front(queue, claimed, count);
       if (!grp.sync()) return;
@@ -1253,6 +1272,42 @@ int solo_lanes(int rows, double mean_len) {
   return std::min(g, lanes_for(mean_len, 1.0));
 }
 
+// CTAs per team (RANKS, 2 RANKS or 4 RANKS) for the batch's team LPs on `ctas`
+// CTAs: the size whose greedy schedule (largest LP first, as the queue is
+// taken) ends first, the smaller one within 5 %.  An iteration of an LP costs a
+// team of s CTAs about 2.3e-3 us per nonzero / s plus 12 us of barriers and
+// reductions.  A batch of thousands keeps teams of four (10.9 s against 11.8
+// with teams of eight for 4096 uneven LPs); where a few large LPs hold the
+// batch up, or the last round of equal ones is nearly empty, larger teams win:
+// 256 uneven LPs, the largest of 2e6 nonzeros, 43.6 ms with teams of four and
+// 24.5 ms for 48 iterations; 48 transportation LPs of 1.2e5 nonzeros 26.2 ms
+// (teams of four on 48 CTAs) and 10.5 ms for 32.
+int plan_team_size(const pdlp_lp *lps, int count, int ctas) {
+  std::vector<double> work;
+  for (int i = 0; i < count; ++i) {
+    const double nnz = lps[i].row_ptr[lps[i].m];
+    if (nnz >= (double)TEAM_MIN_NNZ) work.push_back(nnz);
+  }
+  std::sort(work.begin(), work.end(), std::greater<double>());
+  int best = RANKS;
+  double best_t = INFINITY;
+  for (int s = RANKS; s <= 4 * RANKS && s <= ctas; s *= 2) {
+    std::vector<double> ends(ctas / s, 0.0);  // a heap, earliest first
+    double t = 0.0;
+    for (double w : work) {
+      std::pop_heap(ends.begin(), ends.end(), std::greater<double>());
+      ends.back() += 2.3e-3 * w / s + 12.0;
+      t = std::max(t, ends.back());
+      std::push_heap(ends.begin(), ends.end(), std::greater<double>());
+    }
+    if (t < 0.95 * best_t) {
+      best = s;
+      best_t = t;
+    }
+  }
+  return best;
+}
+
 void free_batch(pdlp_batch *b) {
   if (!b) return;
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
@@ -1274,9 +1329,20 @@ int launch_solve(pdlp_batch *b, const Arrays &A, const Params &p, cudaStream_t s
   BCK(cudaMemsetAsync(b->d_queue, 0, 8 + 4 * (size_t)b->count, s));
   // team barrier counters and the abort flag start at zero
   BCK(cudaMemsetAsync(b->team_words, 0, b->team_words_bytes, s));
-  k_batch_solve<<<b->grid, NTB, RESIDENT_MAX, s>>>(A, b->d_inst, b->d_order, b->count, b->d_queue,
-                                                  b->d_queue + 2, p, (long long)RESIDENT_MAX, b->ts);
-  BCK(cudaGetLastError());
+  // with teams the CTAs wait on one another: all resident or none, whatever
+  // else runs on the GPU
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(b->grid);
+  cfg.blockDim = dim3(NTB);
+  cfg.dynamicSmemBytes = RESIDENT_MAX;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = b->ts.teams > 0 ? 1 : 0;
+  BCK(cudaLaunchKernelEx(&cfg, k_batch_solve, A, (const Inst *)b->d_inst, (const int *)b->d_order, b->count, b->d_queue,
+                         b->d_queue + 2, p, (long long)RESIDENT_MAX, b->ts));
   return PDLP_OK;
 }
 
@@ -1382,10 +1448,15 @@ int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const
     return set_error(PDLP_ERR_CUDA, cudaGetErrorString(e));
   }
   b->grid = std::max(1, std::min(count, per_sm * b->num_sms));
-  // with room for a team: whole teams plus BACK_CTAS CTAs that start from
-  // the small end of the queue
-  const int teams = b->grid >= BACK_CTAS + TEAM ? (b->grid - BACK_CTAS) / TEAM : 0;
-  if (teams) b->grid = teams * TEAM + BACK_CTAS;
+  // a batch of at least BACK_CTAS + RANKS LPs has teams: then every SM works,
+  // in whole teams plus CTAs that start from the small end of the queue (none
+  // of which may take a team's LP)
+  const bool has_teams = b->grid >= BACK_CTAS + RANKS;
+  const int back = b->team_lps ? std::min(BACK_CTAS, count - b->team_lps) : BACK_CTAS;
+  if (has_teams && b->team_lps) b->grid = std::max(b->grid, per_sm * b->num_sms);
+  const int team_size = plan_team_size(lps, count, b->grid - back);
+  const int teams = has_teams ? (b->grid - back) / team_size : 0;
+  if (teams) b->grid = teams * team_size + back;
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   size_t off = 0;
   const size_t o_kptr = off; off += al(4 * KP);
@@ -1407,7 +1478,7 @@ int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const
   const size_t o_or = off; off += al(4 * count);
   const size_t o_q = off; off += al(8 + 4 * (size_t)count);  // front / back counters, claim flags
   const size_t o_tw = off; off += al(4 * (3 * (size_t)teams + 1));
-  const size_t o_tsl = off; off += al(8 * (size_t)std::max(teams, 1) * 2 * TEAM * 16);
+  const size_t o_tsl = off; off += al(8 * (size_t)std::max(teams, 1) * 2 * TEAM_SLOTS);
   b->arena_bytes = off;
   e = cudaMalloc((void **)&b->arena, b->arena_bytes);
   if (e != cudaSuccess) {
@@ -1442,6 +1513,7 @@ int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const
     b->ts.abort = (int *)(w + 3 * teams);
     b->ts.slots = (double *)(Ar + o_tsl);
     b->ts.teams = teams;
+    b->ts.size = team_size;
     b->team_words = w;
     b->team_words_bytes = 4 * (3 * (size_t)teams + 1);
   }
@@ -1702,7 +1774,7 @@ int pdlp_batch_info(const pdlp_batch *b, pdlp_batch_stats *s) {
   s->resident = b->resident;
   s->resident_max_bytes = RESIDENT_MAX;
   s->team_lps = b->ts.teams > 0 ? b->team_lps : 0;
-  s->team_size = TEAM;
+  s->team_size = b->ts.size;
   s->team_min_nnz = (int32_t)TEAM_MIN_NNZ;
   return PDLP_OK;
 }

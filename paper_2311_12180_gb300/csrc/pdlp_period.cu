@@ -131,29 +131,6 @@ struct Barrier {
   }
 };
 
-// Sums of NV (<= 32) values over the warp, transposed: at each level half of
-// the values go to one half of the lanes, so 32 values take 31 additions per
-// lane (5 each without it) and 3 take 6.  Value a ends in the lanes with
-// lane / (32 / NP) == a, NP the next power of two.
-__host__ __device__ constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : 2 * pow2_at_least((n + 1) / 2); }
-
-template <int NV, int W, int OFF>
-__device__ __forceinline__ void butterfly(double (&v)[NV], int lane) {
-  if constexpr (W > 1) {
-    constexpr int H = W / 2;
-    const bool hi = (lane & OFF) != 0;
-#pragma unroll
-    for (int i = 0; i < H && i < NV; ++i) {
-      const double a = v[i], b = i + H < NV ? v[i + H < NV ? i + H : 0] : 0.0;
-      v[i] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, OFF);
-    }
-    if constexpr (OFF > 1) butterfly<NV, H, OFF / 2>(v, lane);
-  } else {
-    v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
-    if constexpr (OFF > 1) butterfly<NV, 1, OFF / 2>(v, lane);
-  }
-}
-
 // ---- the kernels' grids, dealt out over this launch's CTAs ----
 //
 // A multiple of G groups is dealt out whole: a group's eight virtual warps run
