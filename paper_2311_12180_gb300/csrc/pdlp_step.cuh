@@ -59,7 +59,7 @@ __device__ __forceinline__ void strided_dot(const int32_t *__restrict__ ip, cons
 #pragma unroll
       for (int a = 0; a < NV; ++a) {
         const double xv = c[u] >= 0 ? __ldg(xs[a] + c[u]) : 0.0;
-        g[a][u] = SCALED ? sc[a] * xv : xv;
+        g[a][u] = SCALED && (NV == 1 || a > 0) ? sc[a] * xv : xv;
       }
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -72,7 +72,7 @@ __device__ __forceinline__ void strided_dot(const int32_t *__restrict__ ip, cons
 #pragma unroll
     for (int a = 0; a < NV; ++a) {
       const double xv = c >= 0 ? __ldg(xs[a] + c) : 0.0;
-      acc[a] = fma(widen(v), SCALED ? sc[a] * xv : xv, acc[a]);
+      acc[a] = fma(widen(v), SCALED && (NV == 1 || a > 0) ? sc[a] * xv : xv, acc[a]);
     }
   }
 }
@@ -199,7 +199,8 @@ __device__ __forceinline__ void long_flush(LongRows<NV> &lr, Epi &ep) {
 
 // y = A x for NV (1 or 2) gathered vectors, each finished row r passed to
 // ep.finish(r, sums) after ep.prefetch(r).  With SCALED, gathered entries of
-// vector a are multiplied by sc[a] (the epoch average (1/W) sum).  Warp w of
+// vector a are multiplied by sc[a] (the epoch average (1/W) sum); sc[0] of two
+// is 1 and costs no multiply.  Warp w of
 // the grid takes items w, 2G - 1 - w, 2G + w, ... of the schedule (G warps):
 // a snake over the cost-sorted items, so every warp gets about the same work.
 template <int U, typename VT, int NV, bool SCALED, class Epi>
