@@ -22,6 +22,7 @@
 #include "pdlp.h"
 #include "pdlp_host.h"
 #include "pdlp_internal.cuh"
+#include "pdlp_period.cuh"
 #include "pdlp_sell.h"
 #include "pdlp_setup.cuh"
 

@@ -183,7 +183,6 @@ struct PeriodPlan {
 // decides ctas, cluster and share_bytes (p.grids set; items of K and K' in schedule order)
 void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int nk, const int4 *t_items, int nt,
                  int64_t stored, int value_bytes, int num_sms);
-size_t period_part_doubles();
 cudaError_t period_init();
 cudaError_t launch_period(const PeriodPlan &p, const SellMat &K, const SellMat &KT, const Vecs &V, DevState *st,
                           int max_trials, cudaStream_t s);

@@ -46,6 +46,7 @@
 #include <vector>
 
 #include "pdlp_internal.cuh"
+#include "pdlp_period.cuh"
 #include "pdlp_step.cuh"
 
 namespace pdlp {
@@ -130,33 +131,6 @@ struct Barrier {
     return wait();
   }
 };
-
-// ---- the kernels' grids, dealt out over this launch's CTAs ----
-//
-// A multiple of G groups is dealt out whole: a group's eight virtual warps run
-// on one CTA (a snake over the CTAs, as the groups' costs fall), which adds
-// them, and part[a][group] is what the other CTAs read.  The rest, the first
-// and most expensive groups (in a small LP: all of them), is spread by virtual
-// warps, so that every CTA gets the same number of them and the longest rows
-// meet on no scheduler; their sums go to part[a][v], and the totals add a
-// group's eight.
-
-constexpr int MAX_SLOTS = 8;  // whole groups of one CTA
-
-template <bool CLUSTER>
-__host__ __device__ __forceinline__ int spread_groups(int groups, int grid) {
-  return CLUSTER ? groups : groups % grid;
-}
-// round r of a snake over the CTAs: this CTA's turn in it
-__host__ __device__ __forceinline__ int snake(int round, int block, int grid) {
-  return round * grid + ((round & 1) ? grid - 1 - block : block);
-}
-// doubles of nv values' partials
-template <bool CLUSTER>
-__host__ __device__ __forceinline__ size_t partials(int nv, int groups, int grid) {
-  const int sg = spread_groups<CLUSTER>(groups, grid);
-  return (size_t)nv * (8 * sg + groups - sg);
-}
 
 // f(v, slot) for each of the warp's virtual warps; slot < 0: spread.
 template <bool CLUSTER, class F>
@@ -740,12 +714,9 @@ __global__ void __launch_bounds__(PT<CLUSTER>, 1) k_period(const __grid_constant
     if (S.left > max_iter - S.k) S.left = max_iter - S.k;
     if (S.left < 1) S.left = 1;
   }
-  // the partials of each sum have a place of their own: slower CTAs may still
-  // read one phase's while the next phase writes
-  double *const pA = part;
-  double *const pB = pA + partials<CLUSTER>(1, g.primal, (int)gridDim.x), *const pR1 = pB + partials<CLUSTER>(2, g.dual, (int)gridDim.x),
-               *const pR2 = pR1 + partials<CLUSTER>(NV_R1, g.check_primal, (int)gridDim.x),
-               *const pI = pR2 + partials<CLUSTER>(NV_R2, g.check_dual, (int)gridDim.x), *const pR3 = pI + partials<CLUSTER>(NV_I, g.infeas, (int)gridDim.x);
+  const PeriodParts pp = period_parts<CLUSTER>(g, (int)gridDim.x);
+  double *const pB = part + pp.dual, *const pR1 = part + pp.check_primal, *const pR2 = part + pp.check_dual,
+               *const pI = part + pp.infeas, *const pR3 = part + pp.restart;
   WarpShare wk, wt;
   wk.bits = wt.bits = 0;
   if (share_bytes && max_trials > 0 && (sizeof(VT) == 8 || f32)) {
@@ -768,6 +739,7 @@ __global__ void __launch_bounds__(PT<CLUSTER>, 1) k_period(const __grid_constant
   for (int trial = 0; trial < max_trials && !S.pending && S.status == ST_RUNNING; ++trial) {
     double e1f = 0.0, e2 = 0.0, Wn = 0.0, pend = 0.0;
     int pv, psl = 0;
+    double *const pA = part + pp.primal_of(trial);  // a slower CTA may still read the last trial's
     if (tid == PT<CLUSTER> - 32) {  // the step test's factors, by a warp with little else to do
       const long long k = S.k;
       const double p3 = k < V.npw ? __ldg(V.pw + k) : pow((double)(k + 2), -0.3);
@@ -901,8 +873,6 @@ void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int n
   const int64_t most = *std::max_element(bytes.begin(), bytes.end());
   p.share_bytes = most <= PERIOD_SHARE_MAX ? (int)((most + 1023) / 1024 * 1024) : 0;
 }
-
-size_t period_part_doubles() { return (size_t)(NV_A + NV_B + NV_R1 + NV_R2 + NV_I + NV_R3) * PERIOD_PART_GROUPS; }
 
 cudaError_t period_init() {
   cudaError_t e = cudaSuccess;
