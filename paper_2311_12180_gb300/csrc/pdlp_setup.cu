@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(ST) k_scale_rows(const int32_t *__restrict__ p
           if (e0 + 32 * u >= end) break;
           const int key = e0 + 32 * u + lane < end ? l[u] : SCALE_ROWS;
           unsigned long long bits = (unsigned long long)__double_as_longlong(v[u]) & 0x7fffffffffffffffull;
+          if (bits > 0x7ff0000000000000ull) bits = 0;  // a NaN is left out, as fmax does
 #pragma unroll
           for (int k = 1; k < 32; k <<= 1) {
             const unsigned long long ob = __shfl_down_sync(0xffffffffu, bits, k);
