@@ -218,7 +218,9 @@ int pdlp_solve_warm(pdlp_solver *s, const double *x0, const double *y0, double t
  * accepted steps plus one restart / termination check, or stops early once
  * the solve has ended) without waiting; pdlp_poll waits for the enqueued work
  * and returns the status (-1 = still running); pdlp_finish writes the outputs
- * like pdlp_solve and waits. */
+ * like pdlp_solve and waits.  A small LP's period is one kernel whose CTAs meet
+ * at a barrier; where that waits more than 2 s, pdlp_poll, pdlp_finish and the
+ * solve calls return PDLP_ERR_CUDA until the next pdlp_begin or pdlp_set_state. */
 int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, int64_t max_iter);
 int pdlp_run_periods(pdlp_solver *s, int32_t n_periods);
 int pdlp_poll(pdlp_solver *s, int *status, int64_t *iters);

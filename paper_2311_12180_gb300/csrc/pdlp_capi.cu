@@ -93,12 +93,11 @@ struct pdlp_solver {
   int slots = 0;
   PeriodPlan period;             // ctas > 0: a check period is one launch (pdlp_period.cu), else the graph below
   bool ready = false;            // a period can be enqueued
-  PeriodSync *h_sync = nullptr;  // pinned
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
-  DevState *h_st = nullptr;    // pinned: state written by the host before a solve / read after
-  DevState *h_poll = nullptr;  // pinned: two slots of polled state
+  SolverState *h_st = nullptr;    // pinned: state written by the host before a solve / read after
+  SolverState *h_poll = nullptr;  // pinned: two slots of polled state
   double *h_scal = nullptr;    // pinned
   double eta_hat0 = 1.0, omega0 = 1.0, q_norm = 0.0, c_norm = 0.0;
   double setup_ms = 0.0, solve_ms = 0.0, t0 = 0.0;
@@ -197,7 +196,6 @@ void free_solver(pdlp_solver *s) {
   if (s->h_st) cudaFreeHost(s->h_st);
   if (s->h_poll) cudaFreeHost(s->h_poll);
   if (s->h_scal) cudaFreeHost(s->h_scal);
-  if (s->h_sync) cudaFreeHost(s->h_sync);
   if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   delete s;
@@ -348,12 +346,11 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   CKS(cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking));
   CKS(cudaEventCreateWithFlags(&s->ev[0], cudaEventDisableTiming));
   CKS(cudaEventCreateWithFlags(&s->ev[1], cudaEventDisableTiming));
-  CKS(cudaMallocHost((void **)&s->h_st, sizeof(DevState)));
-  CKS(cudaMallocHost((void **)&s->h_poll, 2 * sizeof(DevState)));
+  CKS(cudaMallocHost((void **)&s->h_st, sizeof(SolverState)));
+  CKS(cudaMallocHost((void **)&s->h_poll, 2 * sizeof(SolverState)));
   CKS(cudaMallocHost((void **)&s->h_scal, 8 * sizeof(double)));
-  CKS(cudaMallocHost((void **)&s->h_sync, sizeof(PeriodSync)));
-  std::memset(s->h_st, 0, sizeof(DevState));
-  s->h_st->status = ST_RUNNING;
+  std::memset((void *)s->h_st, 0, sizeof(SolverState));
+  s->h_st->st.status = ST_RUNNING;
 
   // grids: the occupancy bound, at most one warp per work item (the K'
   // grids are set once its layout is known; the occupancy bound sizes the
@@ -391,11 +388,11 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   const size_t o_pA = L.take(8 * (size_t)s->gridA * NV_A), o_pB = L.take(8 * (size_t)s->gridB * NV_B);
   const size_t o_pR1 = L.take(8 * (size_t)s->gridR1 * NV_R1), o_pR2 = L.take(8 * (size_t)s->gridR2 * NV_R2);
   const size_t o_pR3 = L.take(8 * (size_t)s->gridR3 * NV_R3), o_pI = L.take(8 * (size_t)s->gridI * NV_I);
-  const size_t o_st = L.take(sizeof(DevState)), o_tr = L.take(sizeof(TraceRec) * TRACE_CAP);
+  const size_t o_st = L.take(sizeof(SolverState)), o_tr = L.take(sizeof(TraceRec) * TRACE_CAP);
   const size_t o_sc = L.take(8 * (8 + scalars_work_doubles()));
   const long long npw = 1LL << 20;  // exponent factors for the first 2^20 steps (16 MB)
   const size_t o_pw = L.take(16 * (size_t)npw);
-  const size_t o_ps = L.take(sizeof(PeriodSync)), o_pp = L.take(8 * period_part_doubles());
+  const size_t o_pp = L.take(8 * period_part_doubles());
   s->arena_bytes = L.off;
   CKS(cudaMalloc((void **)&s->arena, s->arena_bytes));
   char *A = s->arena;
@@ -422,7 +419,8 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   s->q = VM(0);
   s->work_m = VM(12);
   s->D1 = VM(14);
-  s->st = (DevState *)(A + o_st);
+  SolverState *const state = (SolverState *)(A + o_st);
+  s->st = &state->st;
   s->d_scal = (double *)(A + o_sc);
 
   Vecs &V = s->V;
@@ -470,7 +468,7 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
   V.trace = (TraceRec *)(A + o_tr);
   V.pw = (const double *)(A + o_pw);
   V.npw = npw;
-  s->period.sync = (PeriodSync *)(A + o_ps);
+  s->period.sync = &state->sync;
   s->period.part = (double *)(A + o_pp);
   V.perm_r = s->perm_r;
   V.perm_c = s->perm_c;
@@ -743,6 +741,13 @@ void pdlp_destroy(pdlp_solver *s) {
   free_solver(s);
 }
 
+// Test hook for the grid barrier's limit (environment PDLP_TEST_PERIOD_STALL=1
+// when the state is set up): a CTA of the whole-GPU path leaves at once.
+static int period_stall() {
+  const char *ev = std::getenv("PDLP_TEST_PERIOD_STALL");
+  return ev && ev[0] == '1' ? 1 : 0;
+}
+
 int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, int64_t max_iter) {
   g_err.clear();
   if (!s) return fail(PDLP_ERR_INVALID, "solver is NULL");
@@ -766,8 +771,8 @@ int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, i
     CK(cudaMemcpyAsync(V.ylast, V.y[0], 8 * M, cudaMemcpyDeviceToDevice, st));
   }
   CK(cudaStreamSynchronize(st));  // h_st may still be read by an earlier async copy
-  DevState &h = *s->h_st;
-  std::memset(&h, 0, sizeof(DevState));
+  DevState &h = s->h_st->st;
+  std::memset((void *)s->h_st, 0, sizeof(SolverState));
   h.eta = s->eta_hat0;
   h.omega = s->omega0;
   h.W = 0.0;
@@ -792,7 +797,9 @@ int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, i
   h.use_f32 = s->prm.value_bits == 32 ? 1 : 0;
   h.polish = s->prm.f32_polish ? 1 : 0;
   h.eps_infeas = s->V.qd ? 0.0 : s->prm.eps_infeas;  // the certificates are the LP's
-  CK(cudaMemcpyAsync(s->st, s->h_st, sizeof(DevState), cudaMemcpyHostToDevice, st));
+  // the barrier words start afresh too: an earlier solve's may have run out
+  CK(cudaMemcpyAsync(s->st, s->h_st, sizeof(SolverState), cudaMemcpyHostToDevice, st));
+  s->period.stall = period_stall();
   // KKT(z^{0,0}): K'y, Kx and the pieces of eq. (kkt) at the start point
   if (s->period.ctas) {
     CK(launch_period(s->period, s->K, s->KT, V, s->st, 0, st));
@@ -815,15 +822,22 @@ int pdlp_run_periods(pdlp_solver *s, int32_t n_periods) {
   return PDLP_OK;
 }
 
+// PDLP_ERR_CUDA where a period's grid barrier ran out.  The error stays with
+// the state until the next pdlp_begin or pdlp_set_state writes both anew.
+static int barrier_result(const SolverState &h) {
+  if (!h.sync.error) return PDLP_OK;
+  return fail(PDLP_ERR_CUDA, "a check period timed out at its grid barrier; the results are incomplete");
+}
+
 int pdlp_poll(pdlp_solver *s, int *status, int64_t *iters) {
   g_err.clear();
   if (!s) return fail(PDLP_ERR_INVALID, "solver is NULL");
   CK(cudaSetDevice(s->device));
-  CK(cudaMemcpyAsync(&s->h_poll[0], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaMemcpyAsync(&s->h_poll[0], s->st, sizeof(SolverState), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
-  if (status) *status = s->h_poll[0].status;
-  if (iters) *iters = s->h_poll[0].k;
-  return PDLP_OK;
+  if (status) *status = s->h_poll[0].st.status;
+  if (iters) *iters = s->h_poll[0].st.k;
+  return barrier_result(s->h_poll[0]);
 }
 
 int pdlp_finish(pdlp_solver *s, double *x_out, double *y_out, int *status, int64_t *iters) {
@@ -832,23 +846,16 @@ int pdlp_finish(pdlp_solver *s, double *x_out, double *y_out, int *status, int64
   CK(cudaSetDevice(s->device));
   cudaStream_t st = s->stream;
   CK(launch_output(s->V, s->st, st));
-  CK(cudaMemcpyAsync(s->h_st, s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(s->h_st, s->st, sizeof(SolverState), cudaMemcpyDeviceToHost, st));
   if (x_out) CK(cudaMemcpyAsync(x_out, s->V.xout, 8 * (size_t)s->n, cudaMemcpyDeviceToHost, st));
   if (y_out && s->m) CK(cudaMemcpyAsync(y_out, s->V.yout, 8 * (size_t)s->m, cudaMemcpyDeviceToHost, st));
-  s->h_sync->error = 0;
-  if (s->period.ctas && !s->period.cluster)
-    CK(cudaMemcpyAsync(s->h_sync, s->period.sync, sizeof(PeriodSync), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (s->h_sync->error) {
-    CK(cudaMemsetAsync(s->period.sync, 0, sizeof(PeriodSync), st));
-    CK(cudaStreamSynchronize(st));
-    return fail(PDLP_ERR_CUDA, "a check period timed out at its grid barrier; the results are incomplete");
-  }
+  if (int rc = barrier_result(*s->h_st)) return rc;
   s->solve_ms = now_ms() - s->t0;
   s->have_result = true;
-  s->last_status = s->h_st->status;
-  if (status) *status = s->h_st->status;
-  if (iters) *iters = s->h_st->k;
+  s->last_status = s->h_st->st.status;
+  if (status) *status = s->h_st->st.status;
+  if (iters) *iters = s->h_st->st.k;
   return PDLP_OK;
 }
 
@@ -869,7 +876,7 @@ static int drive(pdlp_solver *s, double *x_out, double *y_out, int *status, int6
     CK(cudaMemcpyAsync(&s->h_poll[nxt], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(s->ev[nxt], st));
     CK(cudaEventSynchronize(s->ev[slot]));
-    if (s->h_poll[slot].status != ST_RUNNING) break;
+    if (s->h_poll[slot].st.status != ST_RUNNING) break;
     if (now_ms() - s->t0 > limit_ms) {
       CK(launch_time_limit(s->st, st));
       break;
@@ -892,7 +899,7 @@ int pdlp_resume(pdlp_solver *s, double *x_out, double *y_out, int *status, int64
   CK(cudaSetDevice(s->device));
   CK(cudaStreamSynchronize(s->stream));
   CK(cudaMemcpy(s->h_st, s->st, sizeof(DevState), cudaMemcpyDeviceToHost));
-  if (s->h_st->status != ST_RUNNING) return pdlp_finish(s, x_out, y_out, status, iters);
+  if (s->h_st->st.status != ST_RUNNING) return pdlp_finish(s, x_out, y_out, status, iters);
   return drive(s, x_out, y_out, status, iters);
 }
 
@@ -926,7 +933,7 @@ int pdlp_time_kernels(pdlp_solver *s, int32_t n_periods, double *ms, int64_t *la
   auto poll = [&](DevState &out) -> int {
     CK(cudaMemcpyAsync(&s->h_poll[0], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    out = s->h_poll[0];
+    out = s->h_poll[0].st;
     return PDLP_OK;
   };
   int rc = PDLP_OK;
@@ -958,7 +965,7 @@ int pdlp_time_kernels(pdlp_solver *s, int32_t n_periods, double *ms, int64_t *la
 int pdlp_get_info(const pdlp_solver *s, pdlp_info *info) {
   g_err.clear();
   if (!s || !info) return fail(PDLP_ERR_INVALID, "null argument");
-  const DevState &h = *s->h_st;
+  const DevState &h = s->h_st->st;
   std::memset(info, 0, sizeof(*info));
   info->status = s->have_result ? h.status : -1;
   info->which = h.which;
@@ -989,7 +996,7 @@ int pdlp_get_trace(const pdlp_solver *s, pdlp_check *trace, int32_t cap, int32_t
   g_err.clear();
   if (!s || (cap > 0 && !trace)) return fail(PDLP_ERR_INVALID, "null argument");
   CK(cudaSetDevice(s->device));
-  const int nt = s->h_st->ntrace;
+  const int nt = s->h_st->st.ntrace;
   if (count) *count = nt;
   // retained: the last TRACE_CAP records, the oldest at index first % TRACE_CAP
   const int kept = nt < TRACE_CAP ? nt : TRACE_CAP, first = nt - kept;
@@ -1168,8 +1175,10 @@ int pdlp_set_state(pdlp_solver *s, const void *buf, size_t bytes) {
   for (int i = 0; i < STATE_NV_M; ++i)
     if ((rc = push(vm[i], s->m, s->h_perm_r))) return rc;
   std::memset(d.cnt, 0, sizeof(d.cnt));
-  *s->h_st = d;
-  CK(cudaMemcpy(s->st, s->h_st, sizeof(DevState), cudaMemcpyHostToDevice));
+  std::memset((void *)s->h_st, 0, sizeof(SolverState));  // the barrier words start afresh
+  s->h_st->st = d;
+  s->period.stall = period_stall();
+  CK(cudaMemcpy(s->st, s->h_st, sizeof(SolverState), cudaMemcpyHostToDevice));
   s->launches = 0;
   s->have_result = false;
   s->last_status = d.status;

@@ -164,6 +164,12 @@ struct PeriodSync {
   unsigned count, base;  // grid barrier: arrivals so far (only grows), their number when a launch starts
   int error;             // 1: a barrier wait ran out
 };
+// The solver state as it lies in device memory and in the host's copies: one
+// transfer sets up or reads both.
+struct SolverState {
+  DevState st;
+  alignas(128) PeriodSync sync;
+};
 constexpr int PERIOD_CLUSTER = 16;
 constexpr int PERIOD_SHARE_MAX = 200 * 1024;
 constexpr int64_t PERIOD_WORK_MAX = 8000000;
@@ -176,6 +182,7 @@ struct PeriodPlan {
   int ctas = 0;         // 0: the LP is solved by the step and check kernels
   bool cluster = false;
   int share_bytes = 0;  // shared memory of a CTA's items of K and K', 0: read from the L2
+  int stall = 0;        // test hook: a CTA that never arrives at the grid barrier
   PeriodGrids grids;
   PeriodSync *sync = nullptr;
   double *part = nullptr;

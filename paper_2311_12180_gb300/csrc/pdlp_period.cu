@@ -686,11 +686,12 @@ template <bool CLUSTER, bool QP, typename VT>
 __global__ void __launch_bounds__(PT<CLUSTER>, 1) k_period(const __grid_constant__ SellMat K, const __grid_constant__ SellMat KT,
                                                   const __grid_constant__ Vecs V, const __grid_constant__ PeriodGrids g,
                                                   DevState *st, PeriodSync *ps, double *part, int max_trials,
-                                                  int share_bytes) {
+                                                  int share_bytes, int stall) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ Scratch sm;
   StepState &S = sm.S;
   if (st->status != ST_RUNNING) return;
+  if (!CLUSTER && stall && blockIdx.x == 1) return;
   const int f32 = st->use_f32, tid = threadIdx.x;
   const bool keep = st->eps_infeas > 0.0, check = st->mode == MODE_CHECK;
   Barrier<CLUSTER> bar{ps, CLUSTER ? 0u : ps->base, &sm.ok};
@@ -902,7 +903,7 @@ cudaError_t launch_period(const PeriodPlan &p, const SellMat &K, const SellMat &
   cfg.attrs = at;
   cfg.numAttrs = 1;
   auto go = [&](auto kernel) {
-    return cudaLaunchKernelEx(&cfg, kernel, K, KT, V, p.grids, st, p.sync, p.part, max_trials, p.share_bytes);
+    return cudaLaunchKernelEx(&cfg, kernel, K, KT, V, p.grids, st, p.sync, p.part, max_trials, p.share_bytes, p.stall);
   };
   if (p.cluster) {
     at[0].id = cudaLaunchAttributeClusterDimension;
