@@ -204,8 +204,8 @@ void free_solver(pdlp_solver *s) {
 // What enqueueing a period needs: nothing for a one-launch period, else the
 // CUDA graph of one check period.
 int build_graph(pdlp_solver *s) {
-  s->ready = true;
-  if (s->period.ctas || s->gexec) return PDLP_OK;
+  s->ready = s->period.ctas || s->gexec;
+  if (s->ready) return PDLP_OK;
   CK(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < s->slots && e == cudaSuccess; ++i) {
@@ -225,6 +225,7 @@ int build_graph(pdlp_solver *s) {
   if (e2 != cudaSuccess) return fail(PDLP_ERR_CUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e2));
   s->graph = g;
   CK(cudaGraphInstantiate(&s->gexec, s->graph, 0));
+  s->ready = true;
   return PDLP_OK;
 }
 

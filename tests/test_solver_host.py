@@ -1,0 +1,46 @@
+"""The solver's host driver (csrc/pdlp_capi.cu) on a stand-in for the CUDA
+runtime, no GPU: what it answers when a call of the runtime fails."""
+
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2311_12180_gb300 import pdlp as P
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def exe(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not found")
+    csrc, here = os.path.join(ROOT, "paper_2311_12180_gb300", "csrc"), os.path.join(ROOT, "tests")
+    tmp = str(tmp_path_factory.mktemp("solver"))
+    flags = ["-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a", "-I", csrc, "-I", os.path.join(ROOT, "include")]
+    objs = []
+    for src, lang in ((os.path.join(here, "cuda_runtime_host.cpp"), []), (os.path.join(here, "solver_host.cpp"), ["-x", "cu"]),
+                      (os.path.join(csrc, "pdlp_capi.cu"), [])):
+        objs.append(os.path.join(tmp, os.path.basename(src) + ".o"))
+        subprocess.run([nvcc, *flags, *lang, "-c", src, "-o", objs[-1]], check=True)
+    out = os.path.join(tmp, "solver_host")
+    subprocess.run([nvcc, "-cudart", "none", *objs, "-lpthread", "-o", out], check=True)
+    return out
+
+
+def _run(exe, scenario):
+    out = subprocess.run([exe, scenario], capture_output=True, text=True, check=True).stdout.strip().split("\n")
+    rows = []
+    for line in out:
+        w = line.split()
+        rows.append((w[0], int(w[1]), {w[i]: int(w[i + 1]) for i in range(2, len(w), 2)}))
+    return rows
+
+
+def test_a_failed_capture_leaves_no_period_to_run(exe):
+    quad, begin, run, begin2, run2 = _run(exe, "capture")
+    assert quad[1] == P.OK and begin[1] == P.ERR_CUDA
+    assert run[1] == P.ERR_INVALID and run[2]["graph"] == 0  # "call pdlp_begin first"
+    assert begin2[1] == P.OK and run2[1] == P.OK and run2[2]["graph"] == 2
