@@ -291,7 +291,8 @@ int pdlp_get_scaling(const pdlp_solver *s, double *D1, double *D2, double *val_s
 typedef struct {
   int64_t K_stored, K_slices, K_long_rows;    /* stored entries (padding included), slices, long rows */
   int64_t KT_stored, KT_slices, KT_long_rows; /* the same for K' */
-  int32_t long_threshold, pad_;
+  int32_t long_threshold;
+  int32_t period_ctas; /* CTAs of the kernel that runs a whole check period (small LPs), 0: step and check kernels */
 } pdlp_layout_info;
 int pdlp_get_layout(const pdlp_solver *s, pdlp_layout_info *info);
 

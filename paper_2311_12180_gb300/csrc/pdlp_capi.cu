@@ -229,11 +229,32 @@ int build_graph(pdlp_solver *s) {
   return PDLP_OK;
 }
 
+// Launches the one-launch period.  Where the runtime refuses it because the
+// stream has too few SMs for CTAs that wait on one another (a green context's
+// or an MPS client's share; nothing has run), the solver goes over to the step
+// and check kernels for good: the same bits, on any number of SMs.
+int try_period(pdlp_solver *s, int max_trials, bool *done) {
+  *done = false;
+  if (!s->period.ctas) return PDLP_OK;
+  const cudaError_t e = launch_period(s->period, s->K, s->KT, s->V, s->st, max_trials, s->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+      e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration) {
+    cudaGetLastError();
+    s->period.ctas = 0;
+    return build_graph(s);
+  }
+  CK(e);
+  *done = true;
+  return PDLP_OK;
+}
+
 // Enqueues one check period.
-cudaError_t enqueue_period(pdlp_solver *s) {
+int enqueue_period(pdlp_solver *s) {
+  bool done;
+  if (int rc = try_period(s, s->slots, &done)) return rc;
+  if (!done) CK(cudaGraphLaunch(s->gexec, s->stream));
   s->launches++;
-  if (s->period.ctas) return launch_period(s->period, s->K, s->KT, s->V, s->st, s->slots, s->stream);
-  return cudaGraphLaunch(s->gexec, s->stream);
+  return PDLP_OK;
 }
 
 int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const double *c, const int32_t *row_ptr,
@@ -595,7 +616,7 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
     {
       s->period.grids = PeriodGrids{s->gridA, s->gridB, s->gridR1, s->gridR2, s->gridI, s->gridR3};
       period_plan(s->period, m, n, LK.items.data(), (int)LK.items.size(), LT.items.data(), (int)LT.items.size(),
-                  LK.total + LT.total, f32 ? 4 : 8, s->num_sms);
+                  LK.total + LT.total, f32 ? 4 : 8, s->num_sms, s->stream);
       const int grc = build_graph(s);
       if (grc) {
         free_solver(s);
@@ -802,9 +823,9 @@ int pdlp_begin(pdlp_solver *s, const double *x0, const double *y0, double tol, i
   CK(cudaMemcpyAsync(s->st, s->h_st, sizeof(SolverState), cudaMemcpyHostToDevice, st));
   s->period.stall = period_stall();
   // KKT(z^{0,0}): K'y, Kx and the pieces of eq. (kkt) at the start point
-  if (s->period.ctas) {
-    CK(launch_period(s->period, s->K, s->KT, V, s->st, 0, st));
-  } else {
+  bool done;
+  if ((rc = try_period(s, 0, &done))) return rc;
+  if (!done) {
     CK(launch_check_primal(s->KT, V, s->st, s->gridR1, st));
     CK(launch_check_dual(s->K, V, s->st, s->gridR2, st));
   }
@@ -819,7 +840,8 @@ int pdlp_run_periods(pdlp_solver *s, int32_t n_periods) {
   g_err.clear();
   if (!s || !s->ready) return fail(PDLP_ERR_INVALID, "call pdlp_begin first");
   CK(cudaSetDevice(s->device));
-  for (int32_t i = 0; i < n_periods; ++i) CK(enqueue_period(s));
+  for (int32_t i = 0; i < n_periods; ++i)
+    if (int rc = enqueue_period(s)) return rc;
   return PDLP_OK;
 }
 
@@ -868,12 +890,12 @@ static int drive(pdlp_solver *s, double *x_out, double *y_out, int *status, int6
   const double limit_ms = s->prm.time_limit_s > 0.0 ? 1000.0 * s->prm.time_limit_s : INFINITY;
   // one period in flight ahead of the one being polled
   int slot = 0;
-  CK(enqueue_period(s));
+  if (int rc = enqueue_period(s)) return rc;
   CK(cudaMemcpyAsync(&s->h_poll[slot], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
   CK(cudaEventRecord(s->ev[slot], st));
   for (;;) {
     const int nxt = slot ^ 1;
-    CK(enqueue_period(s));
+    if (int rc = enqueue_period(s)) return rc;
     CK(cudaMemcpyAsync(&s->h_poll[nxt], s->st, sizeof(DevState), cudaMemcpyDeviceToHost, st));
     CK(cudaEventRecord(s->ev[nxt], st));
     CK(cudaEventSynchronize(s->ev[slot]));
@@ -1225,6 +1247,7 @@ int pdlp_get_layout(const pdlp_solver *s, pdlp_layout_info *info) {
   g_err.clear();
   if (!s || !info) return fail(PDLP_ERR_INVALID, "null argument");
   *info = s->layout;
+  info->period_ctas = s->period.ctas;
   return PDLP_OK;
 }
 

@@ -187,9 +187,9 @@ struct PeriodPlan {
   PeriodSync *sync = nullptr;
   double *part = nullptr;
 };
-// decides ctas, cluster and share_bytes (p.grids set; items of K and K' in schedule order)
+// decides ctas, cluster and share_bytes (p.grids set; items of K and K' in schedule order; s: the solver's stream)
 void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int nk, const int4 *t_items, int nt,
-                 int64_t stored, int value_bytes, int num_sms);
+                 int64_t stored, int value_bytes, int num_sms, cudaStream_t s);
 cudaError_t period_init();
 cudaError_t launch_period(const PeriodPlan &p, const SellMat &K, const SellMat &KT, const Vecs &V, DevState *st,
                           int max_trials, cudaStream_t s);

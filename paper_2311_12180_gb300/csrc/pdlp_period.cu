@@ -831,6 +831,28 @@ __global__ void __launch_bounds__(PT<CLUSTER>, 1) k_period(const __grid_constant
 
 }  // namespace
 
+namespace {
+// grid, block, shared memory and attribute of a plan's launch
+void launch_config(const PeriodPlan &p, cudaStream_t s, cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&at)[1]) {
+  cfg = cudaLaunchConfig_t{};
+  at[0] = cudaLaunchAttribute{};
+  cfg.gridDim = dim3(p.ctas);
+  cfg.blockDim = dim3(p.cluster ? PT<true> : PT<false>);
+  cfg.dynamicSmemBytes = p.share_bytes;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (p.cluster) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = p.ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  } else {  // its CTAs wait on one another: all resident or none
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+}
+}  // namespace
+
 // Which LPs run as one cluster of PERIOD_CLUSTER CTAs and which on the whole
 // GPU: the FP64 instructions of an iteration (one per 32 stored entries, 6 and
 // 9 per 32 rows for the epilogues) take 19 cycles each on an SM; the cluster's
@@ -841,12 +863,16 @@ __global__ void __launch_bounds__(PT<CLUSTER>, 1) k_period(const __grid_constant
 // K', or 0 when that is more than PERIOD_SHARE_MAX: the rest of the SM's 256
 // KB is the L1 that holds a line for every gather in flight.
 //
+// Where a cluster does not fit the SMs that the stream has (a cluster's CTAs
+// share a GPC), the step and check kernels run the LP; too few SMs for the
+// whole-GPU kernel show at its cooperative launch.
+//
 // LPs above PERIOD_WORK_MAX (stored entries of K and K' plus eight per row and
 // column) keep the step and check kernels: 6.4e6 at 2e6 nonzeros of the
 // power-law recipe, where this path takes 0.93 of their time; at 3e6 (9.6e6)
 // an earlier build without resident shares took 1.03.
 void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int nk, const int4 *t_items, int nt,
-                 int64_t stored, int value_bytes, int num_sms) {
+                 int64_t stored, int value_bytes, int num_sms, cudaStream_t s) {
   if (stored + 8 * ((int64_t)m + n) > PERIOD_WORK_MAX) return;
   const PeriodGrids &g = p.grids;
   const double f64 = (double)stored / 32 + 6.0 * n / 32 + 9.0 * m / 32;
@@ -873,6 +899,18 @@ void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int n
   deal(t_items, nt, g.primal);
   const int64_t most = *std::max_element(bytes.begin(), bytes.end());
   p.share_bytes = most <= PERIOD_SHARE_MAX ? (int)((most + 1023) / 1024 * 1024) : 0;
+  if (p.cluster) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at[1];
+    launch_config(p, s, cfg, at);
+    int fit = 0;
+    const cudaError_t e = value_bytes == 4 ? cudaOccupancyMaxActiveClusters(&fit, k_period<true, true, float>, &cfg)
+                                           : cudaOccupancyMaxActiveClusters(&fit, k_period<true, true, double>, &cfg);
+    if (e != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      p.ctas = 0;
+    }
+  }
 }
 
 cudaError_t period_init() {
@@ -894,26 +932,16 @@ cudaError_t period_init() {
 
 cudaError_t launch_period(const PeriodPlan &p, const SellMat &K, const SellMat &KT, const Vecs &V, DevState *st,
                           int max_trials, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
+  cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  cfg.gridDim = dim3(p.ctas);
-  cfg.blockDim = dim3(p.cluster ? PT<true> : PT<false>);
-  cfg.dynamicSmemBytes = p.share_bytes;
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
+  launch_config(p, s, cfg, at);
   auto go = [&](auto kernel) {
     return cudaLaunchKernelEx(&cfg, kernel, K, KT, V, p.grids, st, p.sync, p.part, max_trials, p.share_bytes, p.stall);
   };
   if (p.cluster) {
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = p.ctas;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     if (K.val32) return V.qd ? go(k_period<true, true, float>) : go(k_period<true, false, float>);
     return V.qd ? go(k_period<true, true, double>) : go(k_period<true, false, double>);
   }
-  at[0].id = cudaLaunchAttributeCooperative;  // its CTAs wait on one another: all resident or none
-  at[0].val.cooperative = 1;
   if (K.val32) return V.qd ? go(k_period<false, true, float>) : go(k_period<false, false, float>);
   return V.qd ? go(k_period<false, true, double>) : go(k_period<false, false, double>);
 }

@@ -109,7 +109,7 @@ EXPORTS = (
 
 class pdlp_layout_info(C.Structure):
     _fields_ = [(f, C.c_int64) for f in ("K_stored", "K_slices", "K_long_rows", "KT_stored", "KT_slices",
-                                          "KT_long_rows")] + [("long_threshold", C.c_int32), ("pad_", C.c_int32)]
+                                          "KT_long_rows")] + [("long_threshold", C.c_int32), ("period_ctas", C.c_int32)]
 
 
 class pdlp_lp(C.Structure):
@@ -513,7 +513,7 @@ class Solver:
     def layout(self) -> dict:
         info = pdlp_layout_info()
         _check(lib().pdlp_get_layout(self.h, C.byref(info)))
-        return {f: int(getattr(info, f)) for f, _ in pdlp_layout_info._fields_ if f != "pad_"}
+        return {f: int(getattr(info, f)) for f, _ in pdlp_layout_info._fields_}
 
     @property
     def stream(self) -> int:

@@ -34,7 +34,9 @@ const char *kernel_class_name(int) { return ""; }
 int occupancy_grid(int, int sms) { return 4 * sms; }
 cudaError_t kernels_init() { return cudaSuccess; }
 cudaError_t period_init() { return cudaSuccess; }
-void period_plan(PeriodPlan &p, int32_t, int32_t, const int4 *, int, const int4 *, int, int64_t, int, int) { p.ctas = plan_ctas; }
+void period_plan(PeriodPlan &p, int32_t, int32_t, const int4 *, int, const int4 *, int, int64_t, int, int, cudaStream_t) {
+  p.ctas = plan_ctas;
+}
 cudaError_t launch_period(const PeriodPlan &, const SellMat &, const SellMat &, const Vecs &, DevState *, int, cudaStream_t) {
   n_period += period_error == cudaSuccess;
   return period_error;
@@ -92,6 +94,25 @@ int main(int argc, char **argv) {
     fail_capture = 0;
     show("begin", pdlp_begin(s, nullptr, nullptr, 1e-6, 100));
     show("run", pdlp_run_periods(s, 2));
+    pdlp_destroy(s);
+    return 0;
+  }
+  if (scenario == "refused" || scenario == "refused later" || scenario == "broken") {
+    // a small LP whose one-launch period does not fit the stream's SMs, from
+    // the start or from some launch on; or fails for another reason
+    plan_ctas = 152;
+    pdlp_solver *s = create();
+    if (scenario != "refused later") period_error = scenario == "broken" ? cudaErrorIllegalAddress : cudaErrorCooperativeLaunchTooLarge;
+    show("begin", pdlp_begin(s, nullptr, nullptr, 1e-6, 100));
+    if (scenario == "refused later") period_error = cudaErrorInvalidClusterSize;
+    show("run", pdlp_run_periods(s, 2));
+    int st;
+    int64_t it;
+    double x, y;
+    show("finish", pdlp_finish(s, &x, &y, &st, &it));
+    pdlp_layout_info info;
+    show("layout", pdlp_get_layout(s, &info));
+    show("ctas", info.period_ctas);
     pdlp_destroy(s);
     return 0;
   }

@@ -11,6 +11,8 @@ from paper_2311_12180_gb300 import pdlp as P
 
 pytestmark = pytest.mark.gpu
 
+SMS = 152  # of a GB300
+
 
 def _ragged(m, n, longest, most):
     """Rows of up to `longest` entries among rows of fewer than `most`, and a dense column."""
@@ -29,6 +31,7 @@ def _ragged(m, n, longest, most):
 def test_rejected_trials_equal_the_step_kernels(shape, period):
     N = 400
     with P.Solver(_ragged(*shape), check_period=period) as s:
+        assert s.layout()["period_ctas"] == (16 if shape[0] == 700 else SMS)
         runs = []
         for _ in range(3):
             a = s.solve(tol=1e-14, max_iter=N)

@@ -44,3 +44,16 @@ def test_a_failed_capture_leaves_no_period_to_run(exe):
     assert quad[1] == P.OK and begin[1] == P.ERR_CUDA
     assert run[1] == P.ERR_INVALID and run[2]["graph"] == 0  # "call pdlp_begin first"
     assert begin2[1] == P.OK and run2[1] == P.OK and run2[2]["graph"] == 2
+
+
+@pytest.mark.parametrize("scenario", ["refused", "refused later"])
+def test_a_period_that_does_not_fit_falls_back_to_the_step_kernels(exe, scenario):
+    begin, run, finish, _, ctas = _run(exe, scenario)
+    assert begin[1] == P.OK and run[1] == P.OK and finish[1] == P.OK
+    assert run[2]["graph"] == 2 and ctas[1] == 0
+    assert (begin[2]["check"], begin[2]["period"]) == ((2, 0) if scenario == "refused" else (0, 1))
+
+
+def test_another_launch_error_is_reported(exe):
+    begin, *_, ctas = _run(exe, "broken")
+    assert begin[1] == P.ERR_CUDA and ctas[1] == 152
