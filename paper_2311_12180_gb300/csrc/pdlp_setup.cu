@@ -9,6 +9,7 @@
 
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -28,13 +29,33 @@ __device__ __forceinline__ double warp_add(double v) {
   return v;
 }
 
+// Rows of more than LONG_ROW entries are taken by a warp each, whichever they
+// lie next to; k_long_rows lists them (list[0..), their number in list[rows],
+// zeroed before; the order is of no account).  48: at 96, 1000 rows of 100 take
+// 591 us instead of 289, at 32 30000 rows of 100 take 1733 instead of 1564.
+constexpr int LONG_ROW = 48;
+__global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t rows, int32_t *__restrict__ list) {
+  const int lane = threadIdx.x & 31;
+  for (long long r0 = (long long)blockIdx.x * ST + threadIdx.x - lane; r0 < rows; r0 += (long long)gridDim.x * ST) {
+    const long long r = r0 + lane;
+    const bool is = r < rows && ptr[r + 1] - ptr[r] > LONG_ROW;
+    const unsigned all = __ballot_sync(0xffffffffu, is);
+    int at = 0;
+    if (lane == 0 && all) at = atomicAdd(list + rows, __popc(all));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(all & ((1u << lane) - 1u));
+    if (is) list[at] = (int32_t)r;
+  }
+}
+
 // out[r] = sum_e |val[e]|^p: lane-strided partial sums of a row over 32 lanes,
 // then the xor tree.  A row of at most G entries gives the same sum on G
-// lanes (its other partials are zeros), so a warp takes 32 rows and puts the
-// short ones on G = 1, 8 or 16 lanes: an FP64 addition costs a scheduler 64
-// cycles whatever the number of lanes.
-__global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restrict__ val, int32_t rows,
-                          double *__restrict__ out, double p) {
+// lanes (its other partials are zeros), so a warp takes `per_warp` (at most
+// 32) rows and puts the short ones on G = 1, 8 or 16 lanes: an FP64 addition
+// costs a scheduler 64 cycles whatever the number of lanes.  `longs`: the list
+// of the rows that have a warp to themselves, or null: all rows are taken in
+// turn.
+__global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restrict__ val, int32_t rows, int per_warp,
+                          const int32_t *__restrict__ longs, double *__restrict__ out, double p) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * ST + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * ST) >> 5;
@@ -42,11 +63,23 @@ __global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restr
     const double a = fabs(val[e]);
     return (p == 1.0) ? a : pow(a, p);
   };
-  for (long long r0 = warp * 32; r0 < rows; r0 += nwarps * 32) {
-    const bool in = r0 + lane < rows;
+  if (longs) {
+    const int32_t count = longs[rows];
+    for (long long i = warp; i < count; i += nwarps) {
+      const int32_t r = longs[i];
+      const int b = ptr[r], n = ptr[r + 1] - b;
+      double acc = 0.0;
+      for (unsigned e = lane; e < (unsigned)n; e += 32) acc += term(b + (int)e);
+      acc = warp_add(acc);
+      if (lane == 0) out[r] = acc;
+    }
+  }
+  for (long long r0 = warp * per_warp; r0 < rows; r0 += nwarps * per_warp) {
+    const bool in = lane < per_warp && r0 + lane < rows;
     const int e0 = in ? ptr[r0 + lane] : 0, len = in ? ptr[r0 + lane + 1] - e0 : 0;
+    const bool mine_to_sum = in && !(longs && len > LONG_ROW);
     double sum = len == 1 ? term(e0) : 0.0;
-    unsigned left = __ballot_sync(0xffffffffu, len > 1);
+    unsigned left = __ballot_sync(0xffffffffu, mine_to_sum && len > 1);
     for (int G = 8; G <= 32; G <<= 1) {  // rows of 2-8 entries, four at a time; 9-16, two; longer, one
       unsigned todo = __ballot_sync(0xffffffffu, (left >> lane & 1u) && (len <= G || G == 32));
       left &= ~todo;
@@ -60,7 +93,7 @@ __global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restr
         const int b = __shfl_sync(0xffffffffu, e0, mine & 31), n = __shfl_sync(0xffffffffu, len, mine & 31);
         double acc = 0.0;
         if (mine >= 0)
-          for (int e = lane % G; e < n; e += G) acc += term(b + e);
+          for (unsigned e = lane % G; e < (unsigned)n; e += G) acc += term(b + (int)e);
         for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         // hand the sum to the row's lane
         for (int k = 0; k < 32 / G; ++k) {
@@ -70,27 +103,32 @@ __global__ void k_row_sum(const int32_t *__restrict__ ptr, const double *__restr
         }
       }
     }
-    if (in) out[r0 + lane] = sum;
+    if (mine_to_sum) out[r0 + lane] = sum;
   }
 }
 
-// Rows in storage order, SCALE_ROWS rows a warp: their entries are one
-// contiguous stream, taken 32 lanes x SCALE_U at a time whatever the rows'
-// lengths; an entry's row is found among the starts by shuffles.  SCALE: with
-// the factors r, s of K's rows and columns and their reciprocals,
+// Rows in storage order, SCALE_ROWS rows a warp: the entries between two long
+// rows are one contiguous stream, taken 32 lanes x SCALE_U at a time whatever
+// the rows' lengths; an entry's row is found among the starts by shuffles.  The
+// long rows of the list have a warp each, taken first.  SCALE: with the factors
+// r, s of K's rows and columns and their reciprocals,
 //   K  (KMAJOR):  val[e] = (val[e] / r[row]) / s[idx[e]],
 //   K' (else):    val[e] = (val[e] / r[idx[e]]) / s[row]
 // (div_rn: the correctly rounded quotients).  maxima (may be null): the row
-// maxima of |val| afterwards, as IEEE bits, by a segmented integer maximum:
-// the next Ruiz pass's norms without another pass over the matrix.
-// The FP64 pipe (6 operations an entry) and, on power-law rows, the warp with
-// the most entries bound it: the eleven passes over 3e6 nonzeros take 2.1 ms,
-// 2.7 with 32 rows a warp and one load at a time, 7.5 as warp-per-row passes
-// with plain divisions.
-constexpr int SCALE_ROWS = 8, SCALE_U = 4;
+// maxima of |val| afterwards, as IEEE bits (a NaN left out, as fmax does), by a
+// segmented integer maximum: the next Ruiz pass's norms without another pass
+// over the matrix.
+// Bound by the FP64 pipe (6 operations an entry) and by the loads in flight:
+// four CTAs an SM (64 registers) take 1.77 ms for the eleven passes over 3e6
+// power-law nonzeros, 1.80 with three, 2.02 with two; 7.5 ms as warp-per-row
+// passes with plain divisions.  300 columns of 6000 entries: 1.80 ms, 13.5 with
+// eight of them a warp, 3.8 warp-per-row.  64 rows of 10000 next to one another
+// among 1e5 of 5: 2.6 ms against 8.6.
+constexpr int SCALE_ROWS = 8, SCALE_U = 4, SCALE_CTAS = 4;
 template <bool SCALE, bool KMAJOR>
-__global__ void __launch_bounds__(ST) k_scale_rows(const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
-                                                   double *__restrict__ val, int32_t rows, const double *__restrict__ r,
+__global__ void __launch_bounds__(ST, SCALE_CTAS) k_scale_rows(const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
+                                                   double *__restrict__ val, int32_t rows,
+                                                   const int32_t *__restrict__ longs, const double *__restrict__ r,
                                                    const double *__restrict__ rr, const double *__restrict__ s,
                                                    const double *__restrict__ rs,
                                                    unsigned long long *__restrict__ maxima) {
@@ -99,66 +137,120 @@ __global__ void __launch_bounds__(ST) k_scale_rows(const int32_t *__restrict__ p
   unsigned long long *const mx = smax[threadIdx.x >> 5];
   const long long warp = ((long long)blockIdx.x * ST + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * ST) >> 5;
-  for (long long r0 = warp * SCALE_ROWS; r0 < rows; r0 += nwarps * SCALE_ROWS) {
-    // starts of the warp's rows (lanes 0..SCALE_ROWS - 1) and the end of the last
-    const int start = lane <= SCALE_ROWS ? ptr[min((long long)rows, r0 + lane)] : 0;
-    const int b = __shfl_sync(0xffffffffu, start, 0), end = __shfl_sync(0xffffffffu, start, SCALE_ROWS);
-    if (lane < SCALE_ROWS) mx[lane] = 0;
-    __syncwarp();
-    for (int e0 = b; e0 < end; e0 += 32 * SCALE_U) {
+  auto magnitude = [](double v) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return bits > 0x7ff0000000000000ull ? 0ull : bits;
+  };
+  const int32_t count = longs[rows];
+  for (long long i = warp; i < count; i += nwarps) {
+    const int32_t row = longs[i];
+    const unsigned b = ptr[row], end = ptr[row + 1];
+    const double fa = SCALE ? (KMAJOR ? r : s)[row] : 1.0, fr = SCALE ? (KMAJOR ? rr : rs)[row] : 1.0;
+    unsigned long long most = 0;
+    for (unsigned e0 = b; e0 < end; e0 += 32 * SCALE_U) {
       double v[SCALE_U];
-      int o[SCALE_U], l[SCALE_U];
+      int o[SCALE_U];
 #pragma unroll
       for (int u = 0; u < SCALE_U; ++u) {
-        const int e = min(e0 + 32 * u + lane, end - 1);
+        const unsigned e = min(e0 + 32 * u + lane, end - 1);
         v[u] = val[e];
         o[u] = SCALE ? idx[e] : 0;
       }
-#pragma unroll
-      for (int u = 0; u < SCALE_U; ++u) {
-        const int e = e0 + 32 * u + lane;
-        l[u] = 0;  // the last row that starts at or before e
-#pragma unroll
-        for (int k = SCALE_ROWS / 2; k > 0; k >>= 1)
-          if (__shfl_sync(0xffffffffu, start, l[u] + k) <= e) l[u] += k;
-      }
       if (SCALE) {
-        double a[SCALE_U], ra[SCALE_U], c[SCALE_U], rc[SCALE_U];
+        double c[SCALE_U], rc[SCALE_U];
 #pragma unroll
         for (int u = 0; u < SCALE_U; ++u) {
-          const long long row = min(r0 + l[u], (long long)rows - 1), i = KMAJOR ? row : o[u], j = KMAJOR ? o[u] : row;
-          a[u] = r[i];
-          ra[u] = rr[i];
-          c[u] = s[j];
-          rc[u] = rs[j];
+          c[u] = (KMAJOR ? s : r)[o[u]];
+          rc[u] = (KMAJOR ? rs : rr)[o[u]];
         }
 #pragma unroll
         for (int u = 0; u < SCALE_U; ++u)
           if (e0 + 32 * u < end) {
-            v[u] = div_rn(div_rn(v[u], a[u], ra[u]), c[u], rc[u]);
+            v[u] = KMAJOR ? div_rn(div_rn(v[u], fa, fr), c[u], rc[u]) : div_rn(div_rn(v[u], c[u], rc[u]), fa, fr);
             if (e0 + 32 * u + lane < end) val[e0 + 32 * u + lane] = v[u];
           }
       }
       if (maxima) {
 #pragma unroll
-        for (int u = 0; u < SCALE_U; ++u) {
-          if (e0 + 32 * u >= end) break;
-          const int key = e0 + 32 * u + lane < end ? l[u] : SCALE_ROWS;
-          unsigned long long bits = (unsigned long long)__double_as_longlong(v[u]) & 0x7fffffffffffffffull;
-          if (bits > 0x7ff0000000000000ull) bits = 0;  // a NaN is left out, as fmax does
+        for (int u = 0; u < SCALE_U; ++u)  // past the end: the last entry again, unscaled
+          if (e0 + 32 * u + lane < end) most = max(most, magnitude(v[u]));
+      }
+    }
+    if (maxima) {
+      for (int k = 16; k > 0; k >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, k));
+      if (lane == 0) maxima[row] = most;
+    }
+  }
+  for (long long r0 = warp * SCALE_ROWS; r0 < rows; r0 += nwarps * SCALE_ROWS) {
+    // starts of the warp's rows (lanes 0..SCALE_ROWS - 1) and the end of the last
+    const int start = lane <= SCALE_ROWS ? ptr[min((long long)rows, r0 + lane)] : 0;
+    const int next = __shfl_down_sync(0xffffffffu, start, 1);
+    const unsigned skip = __ballot_sync(0xffffffffu, lane < SCALE_ROWS && next - start > LONG_ROW);
+    if (lane < SCALE_ROWS) mx[lane] = 0;
+    __syncwarp();
+    for (int k0 = 0; k0 < SCALE_ROWS;) {  // rows k0 to k1 - 1: a stream up to the next long row
+      if (skip >> k0 & 1u) {
+        ++k0;
+        continue;
+      }
+      const unsigned ahead = skip >> k0;
+      const int k1 = ahead ? k0 + __ffs(ahead) - 1 : SCALE_ROWS;
+      const unsigned b = __shfl_sync(0xffffffffu, start, k0), end = __shfl_sync(0xffffffffu, start, k1);
+      k0 = k1;
+      for (unsigned e0 = b; e0 < end; e0 += 32 * SCALE_U) {
+        double v[SCALE_U];
+        int o[SCALE_U], l[SCALE_U];
 #pragma unroll
-          for (int k = 1; k < 32; k <<= 1) {
-            const unsigned long long ob = __shfl_down_sync(0xffffffffu, bits, k);
-            const int ok = __shfl_down_sync(0xffffffffu, key, k);
-            if (lane + k < 32 && ok == key && ob > bits) bits = ob;
+        for (int u = 0; u < SCALE_U; ++u) {
+          const unsigned e = min(e0 + 32 * u + lane, end - 1);
+          v[u] = val[e];
+          o[u] = SCALE ? idx[e] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < SCALE_U; ++u) {
+          const unsigned e = e0 + 32 * u + lane;
+          l[u] = 0;  // the last row that starts at or before e
+#pragma unroll
+          for (int k = SCALE_ROWS / 2; k > 0; k >>= 1)
+            if ((unsigned)__shfl_sync(0xffffffffu, start, l[u] + k) <= e) l[u] += k;
+        }
+        if (SCALE) {
+          double a[SCALE_U], ra[SCALE_U], c[SCALE_U], rc[SCALE_U];
+#pragma unroll
+          for (int u = 0; u < SCALE_U; ++u) {
+            const long long row = min(r0 + l[u], (long long)rows - 1), i = KMAJOR ? row : o[u], j = KMAJOR ? o[u] : row;
+            a[u] = r[i];
+            ra[u] = rr[i];
+            c[u] = s[j];
+            rc[u] = rs[j];
           }
-          const int before = __shfl_up_sync(0xffffffffu, key, 1);
-          if (key < SCALE_ROWS && (lane == 0 || before != key) && bits > mx[key]) mx[key] = bits;
-          __syncwarp();
+#pragma unroll
+          for (int u = 0; u < SCALE_U; ++u)
+            if (e0 + 32 * u < end) {
+              v[u] = div_rn(div_rn(v[u], a[u], ra[u]), c[u], rc[u]);
+              if (e0 + 32 * u + lane < end) val[e0 + 32 * u + lane] = v[u];
+            }
+        }
+        if (maxima) {
+#pragma unroll
+          for (int u = 0; u < SCALE_U; ++u) {
+            if (e0 + 32 * u >= end) break;
+            const int key = e0 + 32 * u + lane < end ? l[u] : SCALE_ROWS;
+            unsigned long long bits = magnitude(v[u]);
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+              const unsigned long long ob = __shfl_down_sync(0xffffffffu, bits, k);
+              const int ok = __shfl_down_sync(0xffffffffu, key, k);
+              if (lane + k < 32 && ok == key && ob > bits) bits = ob;
+            }
+            const int before = __shfl_up_sync(0xffffffffu, key, 1);
+            if (key < SCALE_ROWS && (lane == 0 || before != key) && bits > mx[key]) mx[key] = bits;
+            __syncwarp();
+          }
         }
       }
     }
-    if (maxima && lane < SCALE_ROWS && r0 + lane < rows) maxima[r0 + lane] = mx[lane];
+    if (maxima && lane < SCALE_ROWS && r0 + lane < rows && !(skip >> lane & 1u)) maxima[r0 + lane] = mx[lane];
     __syncwarp();
   }
 }
@@ -333,6 +425,29 @@ int grid_for(long long n) {
   return (int)g;
 }
 
+// Warps that the GPU holds at once, about: where a matrix has no more rows, each
+// has one of its own.
+constexpr int FULL_WARPS = 152 * 64;
+// threads for the rows' groups of k_scale_rows and, if long, a warp each
+int scale_grid(long long rows) {
+  return std::max(grid_for(rows * 32 / SCALE_ROWS), std::min(grid_for(32 * rows), FULL_WARPS * 32 / ST));
+}
+// The list of long rows (rows + 1 ints).
+cudaError_t long_rows(const int32_t *ptr, int32_t rows, int32_t *list, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(list + rows, 0, sizeof(int32_t), s);
+  if (e == cudaSuccess) k_long_rows<<<grid_for(rows), ST, 0, s>>>(ptr, rows, list);
+  return e;
+}
+// Row sums: a row a warp while the GPU has the warps (`longs` unused), else 32
+// and the long ones by themselves.
+void row_sums(const int32_t *ptr, const double *val, int32_t rows, const int32_t *longs, double *out, double p,
+              cudaStream_t s) {
+  if (rows <= FULL_WARPS)
+    k_row_sum<<<grid_for(32LL * rows), ST, 0, s>>>(ptr, val, rows, 1, nullptr, out, p);
+  else
+    k_row_sum<<<std::max(grid_for(rows), FULL_WARPS * 32 / ST), ST, 0, s>>>(ptr, val, rows, 32, longs, out, p);
+}
+
 }  // namespace
 
 cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32_t *K_idx, double *K_val,
@@ -343,23 +458,28 @@ cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32
   k_fill<<<grid_for(n), ST, 0, s>>>(D2, n, 1.0);
   unsigned long long *const mm = reinterpret_cast<unsigned long long *>(w.norm_m),
                            *const mn = reinterpret_cast<unsigned long long *>(w.norm_n);
+  cudaError_t e = m > 0 ? long_rows(K_ptr, m, w.long_m, s) : cudaSuccess;
+  if (e == cudaSuccess) e = long_rows(T_ptr, n, w.long_n, s);
+  if (e != cudaSuccess) return e;
+  const int gm = scale_grid(m), gn = scale_grid(n);
   if (ruiz_iters > 0) {  // the first pass's maxima
-    if (m > 0) k_scale_rows<false, true><<<grid_for(4LL * m), ST, 0, s>>>(K_ptr, K_idx, K_val, m, nullptr, nullptr, nullptr, nullptr, mm);
-    k_scale_rows<false, false><<<grid_for(4LL * n), ST, 0, s>>>(T_ptr, T_idx, T_val, n, nullptr, nullptr, nullptr, nullptr, mn);
+    if (m > 0)
+      k_scale_rows<false, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.long_m, nullptr, nullptr, nullptr, nullptr, mm);
+    k_scale_rows<false, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.long_n, nullptr, nullptr, nullptr, nullptr, mn);
   }
   const int passes = ruiz_iters + (pc_alpha >= 0.0 ? 1 : 0);
   for (int it = 0; it < passes; ++it) {
     if (it >= ruiz_iters) {  // Pock-Chambolle: row sums of K and K'
-      if (m > 0) k_row_sum<<<grid_for(m), ST, 0, s>>>(K_ptr, K_val, m, w.norm_m, 2.0 - pc_alpha);
-      k_row_sum<<<grid_for(n), ST, 0, s>>>(T_ptr, T_val, n, w.norm_n, pc_alpha);
+      if (m > 0) row_sums(K_ptr, K_val, m, w.long_m, w.norm_m, 2.0 - pc_alpha, s);
+      row_sums(T_ptr, T_val, n, w.long_n, w.norm_n, pc_alpha, s);
     }
     k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, w.norm_m, w.norm_n, w.f_m, w.f_n, w.rcp_m, w.rcp_n, D1, D2);
     const bool more = it + 1 < ruiz_iters;  // the next pass needs maxima
     if (m > 0)
-      k_scale_rows<true, true><<<grid_for(4LL * m), ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
-                                                          more ? mm : nullptr);
-    k_scale_rows<true, false><<<grid_for(4LL * n), ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
-                                                         more ? mn : nullptr);
+      k_scale_rows<true, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.long_m, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+                                                 more ? mm : nullptr);
+    k_scale_rows<true, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.long_n, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+                                                more ? mn : nullptr);
   }
   return cudaGetLastError();
 }
@@ -383,8 +503,13 @@ cudaError_t setup_scale_perm(int32_t m, int32_t n, int64_t nnz, const int32_t *K
   }
   if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);
   if (pc_alpha >= 0.0) {  // Pock-Chambolle: row sums over K, column sums over K' (fixed order)
-    if (m > 0) k_row_sum<<<grid_for(m), ST, 0, s>>>(K_ptr, K_val, m, work_m, 2.0 - pc_alpha);
-    k_row_sum<<<grid_for(n), ST, 0, s>>>(T_ptr, T_val, n, work_n, pc_alpha);
+    // the lists of long rows in the reciprocals' place, which k_factors writes after
+    int32_t *const lm = reinterpret_cast<int32_t *>(rcp_m), *const ln = reinterpret_cast<int32_t *>(rcp_n);
+    cudaError_t e = m > FULL_WARPS ? long_rows(K_ptr, m, lm, s) : cudaSuccess;
+    if (e == cudaSuccess && n > FULL_WARPS) e = long_rows(T_ptr, n, ln, s);
+    if (e != cudaSuccess) return e;
+    if (m > 0) row_sums(K_ptr, K_val, m, lm, work_m, 2.0 - pc_alpha, s);
+    row_sums(T_ptr, T_val, n, ln, work_n, pc_alpha, s);
     k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, work_m, work_n, work_m, work_n, rcp_m, rcp_n, D1, D2);
     if (nnz > 0) k_scale_entries<<<eg, ST, 0, s>>>(K_idx, rowid, K_val, nnz, work_m, work_n, rcp_m, rcp_n);
     if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);
@@ -857,7 +982,7 @@ cudaError_t setup_permute(int32_t count, const int32_t *perm, const double *src,
 namespace {
 
 constexpr int32_t NOALLOC_MAX_LINES = 1 << 18;  // rows and columns, each
-__device__ __align__(256) double g_scale_scratch[6 * NOALLOC_MAX_LINES];
+__device__ __align__(256) double g_scale_scratch[7 * NOALLOC_MAX_LINES + 32];
 
 constexpr int MAX_DEVICES = 256;
 std::mutex g_scratch_mu;
@@ -898,7 +1023,9 @@ extern "C" int pdlp_scale_device_noalloc(int32_t m, int32_t n, const int32_t *K_
   }
   double *const p = scratch;
   const ScaleWork w{p, p + NOALLOC_MAX_LINES, p + 2 * NOALLOC_MAX_LINES, p + 3 * NOALLOC_MAX_LINES,
-                    p + 4 * NOALLOC_MAX_LINES, p + 5 * NOALLOC_MAX_LINES};
+                    p + 4 * NOALLOC_MAX_LINES, p + 5 * NOALLOC_MAX_LINES,
+                    reinterpret_cast<int32_t *>(p + 6 * NOALLOC_MAX_LINES),
+                    reinterpret_cast<int32_t *>(p + 6 * NOALLOC_MAX_LINES) + NOALLOC_MAX_LINES + 32};
   e = setup_scale(m, n, 0, const_cast<int32_t *>(K_ptr), const_cast<int32_t *>(K_idx), K_val,
                   const_cast<int32_t *>(KT_ptr), const_cast<int32_t *>(KT_idx), KT_val, D1, D2, w,
                   ruiz_iters, pc_alpha, static_cast<cudaStream_t>(stream));

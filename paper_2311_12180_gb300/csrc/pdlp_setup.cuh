@@ -32,9 +32,11 @@ size_t transpose_work_ints(int32_t n, int64_t nnz);
 int transpose_max_segment();
 
 // Sec. 2.2 scaling of K and K' in place (row-wise passes over both).
-// Scratch: the lines' norms, factors and reciprocals (m and n doubles each).
+// Scratch: the lines' norms, factors and reciprocals (m and n doubles each)
+// and the lists of long rows of K and K' (m + 1 and n + 1 ints).
 struct ScaleWork {
   double *norm_m, *norm_n, *f_m, *f_n, *rcp_m, *rcp_n;
+  int32_t *long_m, *long_n;
 };
 cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32_t *K_idx, double *K_val,
                         int32_t *T_ptr, int32_t *T_idx, double *T_val, double *D1, double *D2, const ScaleWork &w,
