@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -93,6 +94,7 @@ struct pdlp_solver {
   int slots = 0;
   PeriodPlan period;             // ctas > 0: a check period is one launch (pdlp_period.cu), else the graph below
   bool ready = false;            // a period can be enqueued
+  bool in_flight = false;        // counted in g_in_flight
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -201,11 +203,9 @@ void free_solver(pdlp_solver *s) {
   delete s;
 }
 
-// What enqueueing a period needs: nothing for a one-launch period, else the
-// CUDA graph of one check period.
-int build_graph(pdlp_solver *s) {
-  s->ready = s->period.ctas || s->gexec;
-  if (s->ready) return PDLP_OK;
+// The CUDA graph of one check period, of the step and check kernels.
+int capture_graph(pdlp_solver *s) {
+  if (s->gexec) return PDLP_OK;
   CK(cudaStreamBeginCapture(s->cap_stream, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < s->slots && e == cudaSuccess; ++i) {
@@ -225,8 +225,33 @@ int build_graph(pdlp_solver *s) {
   if (e2 != cudaSuccess) return fail(PDLP_ERR_CUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e2));
   s->graph = g;
   CK(cudaGraphInstantiate(&s->gexec, s->graph, 0));
+  return PDLP_OK;
+}
+
+// What enqueueing a period needs: nothing yet for a one-launch period, else
+// the graph.
+int build_graph(pdlp_solver *s) {
+  s->ready = false;
+  if (!s->period.ctas)
+    if (int rc = capture_graph(s)) return rc;
   s->ready = true;
   return PDLP_OK;
+}
+
+// Solvers of each device that have work enqueued which the host has not yet
+// waited for.  A whole-GPU period holds every SM, so solvers on several streams
+// would take turns, where the step kernels of small LPs share the GPU: four LPs
+// of 1e5 nonzeros take 7.9 us an iteration each as step kernels and 14.7 as
+// whole-GPU periods (alone 29.7 and 15.1), sixteen 3.1 and 14.8; two of 1e6
+// 23.7 and 30.2.  So such a period runs while its solver is the only one; its
+// results are the step kernels' bits, whichever run.  (A cluster leaves room
+// for eight others: sixteen solvers of 2e4 nonzeros take 1.6 us, 2.7 as step
+// kernels.)
+std::atomic<int> g_in_flight[64];
+
+void mark_in_flight(pdlp_solver *s, bool on) {
+  if (s->in_flight != on) g_in_flight[s->device % 64] += on ? 1 : -1;
+  s->in_flight = on;
 }
 
 // Launches the one-launch period.  Where the runtime refuses it because the
@@ -235,7 +260,8 @@ int build_graph(pdlp_solver *s) {
 // and check kernels for good: the same bits, on any number of SMs.
 int try_period(pdlp_solver *s, int max_trials, bool *done) {
   *done = false;
-  if (!s->period.ctas) return PDLP_OK;
+  mark_in_flight(s, true);
+  if (!s->period.ctas || (!s->period.cluster && g_in_flight[s->device % 64] > 1)) return PDLP_OK;
   const cudaError_t e = launch_period(s->period, s->K, s->KT, s->V, s->st, max_trials, s->stream);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
       e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration) {
@@ -252,7 +278,10 @@ int try_period(pdlp_solver *s, int max_trials, bool *done) {
 int enqueue_period(pdlp_solver *s) {
   bool done;
   if (int rc = try_period(s, s->slots, &done)) return rc;
-  if (!done) CK(cudaGraphLaunch(s->gexec, s->stream));
+  if (!done) {
+    if (int rc = capture_graph(s)) return rc;
+    CK(cudaGraphLaunch(s->gexec, s->stream));
+  }
   s->launches++;
   return PDLP_OK;
 }
@@ -760,6 +789,7 @@ void pdlp_destroy(pdlp_solver *s) {
   if (!s) return;
   cudaSetDevice(s->device);
   cudaStreamSynchronize(s->stream);
+  mark_in_flight(s, false);
   free_solver(s);
 }
 
@@ -858,6 +888,7 @@ int pdlp_poll(pdlp_solver *s, int *status, int64_t *iters) {
   CK(cudaSetDevice(s->device));
   CK(cudaMemcpyAsync(&s->h_poll[0], s->st, sizeof(SolverState), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
+  mark_in_flight(s, false);
   if (status) *status = s->h_poll[0].st.status;
   if (iters) *iters = s->h_poll[0].st.k;
   return barrier_result(s->h_poll[0]);
@@ -873,6 +904,7 @@ int pdlp_finish(pdlp_solver *s, double *x_out, double *y_out, int *status, int64
   if (x_out) CK(cudaMemcpyAsync(x_out, s->V.xout, 8 * (size_t)s->n, cudaMemcpyDeviceToHost, st));
   if (y_out && s->m) CK(cudaMemcpyAsync(y_out, s->V.yout, 8 * (size_t)s->m, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  mark_in_flight(s, false);
   if (int rc = barrier_result(*s->h_st)) return rc;
   s->solve_ms = now_ms() - s->t0;
   s->have_result = true;
@@ -1186,6 +1218,7 @@ int pdlp_set_state(pdlp_solver *s, const void *buf, size_t bytes) {
   std::vector<double> tmp((size_t)std::max(s->n, s->m));
   cudaStream_t st = s->stream;
   CK(cudaStreamSynchronize(st));
+  mark_in_flight(s, false);
   auto push = [&](double *dst, int32_t count, const std::vector<int32_t> &perm) -> int {
     if (count == 0) return PDLP_OK;
     for (int32_t r = 0; r < count; ++r) tmp[r] = src[perm[r]];
@@ -1219,6 +1252,7 @@ int pdlp_set_quadratic(pdlp_solver *s, const double *qdiag) {
                                           std::to_string(j) + ")");
   CK(cudaSetDevice(s->device));
   CK(cudaStreamSynchronize(s->stream));
+  mark_in_flight(s, false);
   // the captured graph holds the kernels' arguments: rebuilt at the next begin
   s->ready = false;
   if (s->gexec) {

@@ -14,6 +14,7 @@
 
 extern int fail_capture, capturing, n_graph;     // of the runtime's stand-in
 static int plan_ctas = 0;                        // what period_plan decides
+static bool plan_cluster = false;
 static cudaError_t period_error = cudaSuccess;   // of launch_period
 static int n_period = 0, n_check = 0, n_step = 0;  // launches
 
@@ -36,6 +37,7 @@ cudaError_t kernels_init() { return cudaSuccess; }
 cudaError_t period_init() { return cudaSuccess; }
 void period_plan(PeriodPlan &p, int32_t, int32_t, const int4 *, int, const int4 *, int, int64_t, int, int, cudaStream_t) {
   p.ctas = plan_ctas;
+  p.cluster = plan_cluster;
 }
 cudaError_t launch_period(const PeriodPlan &, const SellMat &, const SellMat &, const Vecs &, DevState *, int, cudaStream_t) {
   n_period += period_error == cudaSuccess;
@@ -114,6 +116,32 @@ int main(int argc, char **argv) {
     show("layout", pdlp_get_layout(s, &info));
     show("ctas", info.period_ctas);
     pdlp_destroy(s);
+    return 0;
+  }
+  if (scenario == "several") {  // whole-GPU periods only while a solver is the only one with work in flight
+    plan_ctas = 152;
+    pdlp_solver *a = create(), *b = create();
+    int st;
+    int64_t it;
+    double x, y;
+    show("begin_a", pdlp_begin(a, nullptr, nullptr, 1e-6, 100));
+    show("run_a", pdlp_run_periods(a, 1));
+    show("begin_b", pdlp_begin(b, nullptr, nullptr, 1e-6, 100));
+    show("run_b", pdlp_run_periods(b, 1));
+    show("run_a", pdlp_run_periods(a, 1));
+    show("finish_a", pdlp_finish(a, &x, &y, &st, &it));
+    show("run_b", pdlp_run_periods(b, 1));
+    show("poll_b", pdlp_poll(b, &st, &it));
+    show("run_a", pdlp_run_periods(a, 1));
+    show("run_b", pdlp_run_periods(b, 1));
+    pdlp_destroy(a);
+    show("run_b", pdlp_run_periods(b, 1));
+    plan_cluster = true;  // a cluster leaves room: always its own launch
+    pdlp_solver *c = create();
+    show("begin_c", pdlp_begin(c, nullptr, nullptr, 1e-6, 100));
+    show("run_c", pdlp_run_periods(c, 1));
+    pdlp_destroy(b);
+    pdlp_destroy(c);
     return 0;
   }
   return 2;

@@ -57,3 +57,15 @@ def test_a_period_that_does_not_fit_falls_back_to_the_step_kernels(exe, scenario
 def test_another_launch_error_is_reported(exe):
     begin, *_, ctas = _run(exe, "broken")
     assert begin[1] == P.ERR_CUDA and ctas[1] == 152
+
+
+def test_several_solvers_share_the_gpu_as_step_kernels(exe):
+    rows = _run(exe, "several")
+    assert all(r[1] == P.OK for r in rows)
+    got = [(r[0], r[2]["graph"], r[2]["period"]) for r in rows]
+    assert got == [("begin_a", 0, 1), ("run_a", 0, 2),                   # a alone
+                   ("begin_b", 0, 2), ("run_b", 1, 2), ("run_a", 2, 2),  # both in flight
+                   ("finish_a", 2, 2), ("run_b", 2, 3), ("poll_b", 2, 3),  # b alone
+                   ("run_a", 2, 4), ("run_b", 3, 4),                     # a alone, then both
+                   ("run_b", 3, 5),                                      # a destroyed
+                   ("begin_c", 3, 6), ("run_c", 3, 7)]                   # a cluster beside b
