@@ -233,7 +233,7 @@ struct TeamState {
   int *q;               // queue position broadcast by the team leader
   double *slots;        // [team][2][TEAM_SLOTS] partial sums
   int *abort;           // set when a barrier wait times out
-  int teams, size;      // CTAs per team: RANKS, 2 RANKS or 4 RANKS
+  int teams, size;      // CTAs per team: RANKS, 2 RANKS or 4 RANKS; 1 in a batch without large LPs
 };
 constexpr int RANKS = 4;                     // virtual ranks of a team: its sums' order (see Team)
 constexpr int TEAM_SLOTS = RANKS * 16 * NWB;  // 16 values of every virtual warp
@@ -1159,7 +1159,8 @@ __device__ __forceinline__ int claim_back(const Arrays &A, const Inst *__restric
 // TEAM_MIN_NNZ nonzeros, all its CTAs solve it together, so one large LP
 // that needs many iterations no longer holds a single SM for the whole
 // batch; from the first smaller LP on, the team disbands and each of its
-// CTAs claims LPs alone.  The remaining CTAs start alone from the back, on
+// CTAs claims LPs alone (a batch without such LPs has teams of one).  The
+// remaining CTAs start alone from the back, on
 // the smallest LPs: those need the most iterations, and starting them first
 // keeps them off the end of the schedule.  Large LPs are always solved by a
 // team and small ones always by one CTA, so results do not depend on timing.
@@ -1329,8 +1330,8 @@ int launch_solve(pdlp_batch *b, const Arrays &A, const Params &p, cudaStream_t s
   BCK(cudaMemsetAsync(b->d_queue, 0, 8 + 4 * (size_t)b->count, s));
   // team barrier counters and the abort flag start at zero
   BCK(cudaMemsetAsync(b->team_words, 0, b->team_words_bytes, s));
-  // with teams the CTAs wait on one another: all resident or none, whatever
-  // else runs on the GPU
+  // CTAs of a team wait on one another: all resident or none, whatever else
+  // runs on the GPU
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;
@@ -1340,7 +1341,7 @@ int launch_solve(pdlp_batch *b, const Arrays &A, const Params &p, cudaStream_t s
   cfg.dynamicSmemBytes = RESIDENT_MAX;
   cfg.stream = s;
   cfg.attrs = &at;
-  cfg.numAttrs = b->ts.teams > 0 ? 1 : 0;
+  cfg.numAttrs = b->ts.teams > 0 && b->ts.size > 1 ? 1 : 0;
   BCK(cudaLaunchKernelEx(&cfg, k_batch_solve, A, (const Inst *)b->d_inst, (const int *)b->d_order, b->count, b->d_queue,
                          b->d_queue + 2, p, (long long)RESIDENT_MAX, b->ts));
   return PDLP_OK;
@@ -1447,16 +1448,24 @@ int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const
     free_batch(b);
     return set_error(PDLP_ERR_CUDA, cudaGetErrorString(e));
   }
-  b->grid = std::max(1, std::min(count, per_sm * b->num_sms));
-  // a batch of at least BACK_CTAS + RANKS LPs has teams: then every SM works,
-  // in whole teams plus CTAs that start from the small end of the queue (none
-  // of which may take a team's LP)
-  const bool has_teams = b->grid >= BACK_CTAS + RANKS;
-  const int back = b->team_lps ? std::min(BACK_CTAS, count - b->team_lps) : BACK_CTAS;
-  if (has_teams && b->team_lps) b->grid = std::max(b->grid, per_sm * b->num_sms);
-  const int team_size = plan_team_size(lps, count, b->grid - back);
-  const int teams = has_teams ? (b->grid - back) / team_size : 0;
-  if (teams) b->grid = teams * team_size + back;
+  // A batch of at least BACK_CTAS + RANKS LPs with large ones among them has
+  // teams, and its other CTAs start from the small end of the queue (none of
+  // them may take a team's LP); it holds no more SMs than it has teams and
+  // small LPs to put there.  Without large LPs nobody waits for anybody.
+  const int ctas = per_sm * b->num_sms, small_lps = count - b->team_lps;
+  b->grid = std::max(1, std::min(count, ctas));
+  int teams = 0, team_size = RANKS;
+  if (b->grid >= BACK_CTAS + RANKS) {
+    if (b->team_lps) {
+      const int back = std::min(BACK_CTAS, small_lps);
+      team_size = plan_team_size(lps, count, ctas - back);
+      teams = std::min((ctas - back) / team_size, b->team_lps);
+      b->grid = teams * team_size + std::min(ctas - teams * team_size, small_lps);
+    } else {
+      team_size = 1;
+      teams = b->grid - BACK_CTAS;
+    }
+  }
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   size_t off = 0;
   const size_t o_kptr = off; off += al(4 * KP);
@@ -1774,7 +1783,7 @@ int pdlp_batch_info(const pdlp_batch *b, pdlp_batch_stats *s) {
   s->resident = b->resident;
   s->resident_max_bytes = RESIDENT_MAX;
   s->team_lps = b->ts.teams > 0 ? b->team_lps : 0;
-  s->team_size = b->ts.size;
+  s->team_size = std::max(b->ts.size, RANKS);
   s->team_min_nnz = (int32_t)TEAM_MIN_NNZ;
   return PDLP_OK;
 }
