@@ -1326,6 +1326,22 @@ void free_batch(pdlp_batch *b) {
     if (e_ != cudaSuccess) return set_error(PDLP_ERR_CUDA, (std::string(#call) + ": " + cudaGetErrorString(e_)).c_str()); \
   } while (0)
 
+// Half the teams and single CTAs, at the end one team of the smallest size:
+// for a stream with fewer SMs than the GPU (a green context, an MPS share).
+// The results do not depend on it.  False: nothing less to be had.
+bool shrink_grid(pdlp_batch *b) {
+  TeamState &t = b->ts;
+  const int singles = b->grid - t.teams * t.size;
+  if (t.teams > 1)
+    t.teams /= 2;
+  else if (t.size > RANKS)
+    t.size = RANKS;
+  else if (singles == 0)
+    return false;
+  b->grid = t.teams * t.size + singles / 2;
+  return true;
+}
+
 int launch_solve(pdlp_batch *b, const Arrays &A, const Params &p, cudaStream_t s) {
   BCK(cudaMemsetAsync(b->d_queue, 0, 8 + 4 * (size_t)b->count, s));
   // team barrier counters and the abort flag start at zero
@@ -1336,15 +1352,22 @@ int launch_solve(pdlp_batch *b, const Arrays &A, const Params &p, cudaStream_t s
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(b->grid);
   cfg.blockDim = dim3(NTB);
   cfg.dynamicSmemBytes = RESIDENT_MAX;
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = b->ts.teams > 0 && b->ts.size > 1 ? 1 : 0;
-  BCK(cudaLaunchKernelEx(&cfg, k_batch_solve, A, (const Inst *)b->d_inst, (const int *)b->d_order, b->count, b->d_queue,
-                         b->d_queue + 2, p, (long long)RESIDENT_MAX, b->ts));
-  return PDLP_OK;
+  for (;;) {
+    cfg.gridDim = dim3(b->grid);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_batch_solve, A, (const Inst *)b->d_inst, (const int *)b->d_order,
+                                             b->count, b->d_queue, b->d_queue + 2, p, (long long)RESIDENT_MAX, b->ts);
+    if (e == cudaErrorCooperativeLaunchTooLarge && shrink_grid(b)) {
+      cudaGetLastError();
+      continue;
+    }
+    BCK(e);
+    return PDLP_OK;
+  }
 }
 
 }  // namespace

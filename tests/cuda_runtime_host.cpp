@@ -1,6 +1,7 @@
-// A stand-in for the CUDA runtime calls of csrc/pdlp_capi.cu, for host tests
-// (tests/test_solver_host.py): memory is the host's, streams and events are
-// nothing, graph launches are counted, and a capture fails on request.
+// A stand-in for the CUDA runtime calls of csrc/pdlp_capi.cu and
+// csrc/pdlp_batch.cu, for host tests (tests/test_solver_host.py): memory is the host's, streams and events are
+// nothing, launches run no kernel and are counted, and a capture or a
+// cooperative launch fails on request.
 #include <cuda_runtime_api.h>
 
 #include <cstdio>
@@ -9,6 +10,8 @@
 
 int fail_capture = 0;          // cudaStreamEndCapture fails
 int capturing = 0, n_graph = 0;  // between begin and end of a capture; graph launches
+int resident_ctas = 1 << 30;     // a cooperative launch of more is refused
+int n_launch = 0, last_grid = 0;  // launches by cudaLaunchKernelEx, the last one's CTAs
 
 extern "C" {
 void **__cudaRegisterFatBinary(void *) {
@@ -57,6 +60,24 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
   *g = fail_capture ? nullptr : (cudaGraph_t)(size_t)1;
   return fail_capture ? cudaErrorStreamCaptureInvalidated : cudaSuccess;
 }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *, void **) {
+  for (unsigned i = 0; i < c->numAttrs; ++i)
+    if (c->attrs[i].id == cudaLaunchAttributeCooperative && c->attrs[i].val.cooperative && (int)c->gridDim.x > resident_ctas)
+      return cudaErrorCooperativeLaunchTooLarge;
+  ++n_launch;
+  last_grid = (int)c->gridDim.x;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned) {
+  return *n = 1, cudaSuccess;
+}
+// what nvcc's host code of a file with kernels calls
+void __cudaRegisterFunction(void **, const char *, char *, const char *, int, void *, void *, void *, void *, int *) {}
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, cudaStream_t) { return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
+cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *) { return *k = nullptr, cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **, size_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = nullptr, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }

@@ -12,26 +12,43 @@ from paper_2311_12180_gb300 import pdlp as P
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.fixture(scope="module")
-def exe(tmp_path_factory):
+def _build(out, *sources):
+    """sources: (file, "cu" or "" to compile as its suffix says), or an object file."""
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not found")
-    csrc, here = os.path.join(ROOT, "paper_2311_12180_gb300", "csrc"), os.path.join(ROOT, "tests")
-    tmp = str(tmp_path_factory.mktemp("solver"))
+    csrc = os.path.join(ROOT, "paper_2311_12180_gb300", "csrc")
     flags = ["-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a", "-I", csrc, "-I", os.path.join(ROOT, "include")]
     objs = []
-    for src, lang in ((os.path.join(here, "cuda_runtime_host.cpp"), []), (os.path.join(here, "solver_host.cpp"), ["-x", "cu"]),
-                      (os.path.join(csrc, "pdlp_capi.cu"), [])):
-        objs.append(os.path.join(tmp, os.path.basename(src) + ".o"))
-        subprocess.run([nvcc, *flags, *lang, "-c", src, "-o", objs[-1]], check=True)
-    out = os.path.join(tmp, "solver_host")
+    for src, lang in sources:
+        if src.endswith(".o"):
+            objs.append(src)
+            continue
+        objs.append(os.path.join(os.path.dirname(out), os.path.basename(src) + ".o"))
+        subprocess.run([nvcc, *flags, *(["-x", lang] if lang else []), "-c", src, "-o", objs[-1]], check=True)
     subprocess.run([nvcc, "-cudart", "none", *objs, "-lpthread", "-o", out], check=True)
     return out
 
 
-def _run(exe, scenario):
-    out = subprocess.run([exe, scenario], capture_output=True, text=True, check=True).stdout.strip().split("\n")
+@pytest.fixture(scope="module")
+def exe(tmp_path_factory):
+    here, csrc = os.path.join(ROOT, "tests"), os.path.join(ROOT, "paper_2311_12180_gb300", "csrc")
+    return _build(str(tmp_path_factory.mktemp("solver") / "solver_host"), (os.path.join(here, "cuda_runtime_host.cpp"), ""),
+                  (os.path.join(here, "solver_host.cpp"), "cu"), (os.path.join(csrc, "pdlp_capi.cu"), ""))
+
+
+@pytest.fixture(scope="module")
+def batch_exe(tmp_path_factory):
+    from paper_2311_12180_gb300 import _build as B
+
+    B.build()
+    here = os.path.join(ROOT, "tests")
+    return _build(str(tmp_path_factory.mktemp("batch") / "batch_host"), (os.path.join(here, "cuda_runtime_host.cpp"), ""),
+                  (os.path.join(here, "batch_host.cpp"), "cu"), (os.path.join(B.OBJDIR, "pdlp_batch.cu.o"), ""))
+
+
+def _run(exe, *args):
+    out = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, check=True).stdout.strip().split("\n")
     rows = []
     for line in out:
         w = line.split()
@@ -69,3 +86,18 @@ def test_several_solvers_share_the_gpu_as_step_kernels(exe):
                    ("run_a", 2, 4), ("run_b", 3, 4),                     # a alone, then both
                    ("run_b", 3, 5),                                      # a destroyed
                    ("begin_c", 3, 6), ("run_c", 3, 7)]                   # a cluster beside b
+
+
+@pytest.mark.parametrize("resident,small,large", [(152, 60, 40), (100, 60, 40), (40, 60, 40), (16, 60, 40), (20, 30, 1),
+                                                  (4, 30, 1), (10, 170, 0)])
+def test_a_batch_fits_its_grid_to_the_stream(batch_exe, resident, small, large):
+    """Launches that the runtime refuses as too large are repeated with fewer
+    teams, in create (which times short solves) and in solve; a batch without
+    large LPs has no CTAs that must be resident together."""
+    create, solve = _run(batch_exe, resident, small, large)
+    assert create[1] == P.OK and solve[1] == P.OK
+    assert solve[2]["grid"] == create[2]["grid"] > 0
+    if large:
+        assert resident / 4 < create[2]["grid"] <= resident or create[2]["grid"] == 4 <= resident
+    else:
+        assert create[2]["grid"] == 152
