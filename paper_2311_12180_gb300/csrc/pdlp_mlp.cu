@@ -675,6 +675,7 @@ struct HostCopy {
   char *pinned = nullptr;  // two chunks a thread
   cudaStream_t st[COPY_THREADS] = {};
   cudaEvent_t ready = nullptr;
+  bool tried = false;
 };
 
 struct pdlp_mlp {
@@ -763,17 +764,22 @@ cudaError_t copy_chunks(const HostCopy &hc, int device, int t, char *dst, const 
   return e != cudaSuccess ? e : d;
 }
 
-// The pinned chunks and streams of copy_out, for a net whose results can be
-// large.  Without page-locked memory to be had its copies are plain ones.
+// The pinned chunks and streams of copy_out, made at a net's first large
+// prediction into pageable memory (0.4 ms; a net that only trains has none).
+// Without page-locked memory to be had its copies are plain ones.
 void host_copy_init(pdlp_mlp *M) {
   HostCopy &hc = M->hc;
-  if (sizeof(float) * (size_t)M->maxb * M->out < COPY_MIN) return;
-  cudaError_t e = cudaEventCreateWithFlags(&hc.ready, cudaEventDisableTiming);
+  if (hc.tried) return;
+  hc.tried = true;
+  char *p = nullptr;
+  cudaError_t e = cudaMallocHost((void **)&p, 2 * COPY_THREADS * COPY_CHUNK);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&hc.ready, cudaEventDisableTiming);
   for (int t = 0; t < COPY_THREADS && e == cudaSuccess; ++t)
     e = cudaStreamCreateWithFlags(&hc.st[t], cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&hc.pinned, 2 * COPY_THREADS * COPY_CHUNK);
-  if (e != cudaSuccess) {
-    hc.pinned = nullptr;
+  if (e == cudaSuccess) {
+    hc.pinned = p;
+  } else {
+    if (p) cudaFreeHost(p);
     cudaGetLastError();
   }
 }
@@ -790,13 +796,14 @@ int copy_out(pdlp_mlp *M, float *dst, const float *src, size_t count) {
   const size_t bytes = sizeof(float) * count;
   cudaPointerAttributes pa{};
   const HostCopy &hc = M->hc;
-  bool staged = hc.pinned && bytes >= COPY_MIN;
+  bool staged = bytes >= COPY_MIN;
   if (staged && cudaPointerGetAttributes(&pa, dst) != cudaSuccess) {
     cudaGetLastError();
     staged = false;
   }
   staged = staged && pa.type == cudaMemoryTypeUnregistered;
-  if (!staged) {
+  if (staged) host_copy_init(M);
+  if (!staged || !hc.pinned) {
     MCK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, M->stream));
     return PDLP_OK;
   }
@@ -1042,7 +1049,6 @@ int pdlp_mlp_create(pdlp_mlp **out, int32_t in_dim, int32_t hidden, int32_t out_
   cudaMemsetAsync(M->m2, 0, sizeof(float) * M->nparam, M->stream);
   cudaMemsetAsync(M->p, 0, sizeof(float) * M->nparam, M->stream);
   cudaMemsetAsync(M->err, 0, sizeof(int), M->stream);
-  host_copy_init(M);
   // identity standardisation until data is set
   std::vector<float> zeros(out_dim, 0.0f), ones(out_dim, 1.0f);
   cudaMemcpyAsync(M->mu, zeros.data(), sizeof(float) * out_dim, cudaMemcpyHostToDevice, M->stream);

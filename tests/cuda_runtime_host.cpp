@@ -1,5 +1,5 @@
-// A stand-in for the CUDA runtime calls of csrc/pdlp_capi.cu and
-// csrc/pdlp_batch.cu, for host tests (tests/test_solver_host.py): memory is the host's, streams and events are
+// A stand-in for the CUDA runtime calls of csrc/pdlp_capi.cu, pdlp_batch.cu and
+// pdlp_mlp.cu, for host tests (tests/test_solver_host.py): memory is the host's, streams and events are
 // nothing, launches run no kernel and are counted, and a capture or a
 // cooperative launch fails on request.
 #include <cuda_runtime_api.h>
@@ -11,6 +11,8 @@
 int fail_capture = 0;          // cudaStreamEndCapture fails
 int capturing = 0, n_graph = 0;  // between begin and end of a capture; graph launches
 int resident_ctas = 1 << 30;     // a cooperative launch of more is refused
+int n_pinned = 0, n_streams = 0, fail_pinned = 0;  // calls of cudaMallocHost and cudaStreamCreateWithFlags
+const void *page_locked = nullptr;                 // this address is page-locked memory, all others are pageable
 int n_launch = 0, last_grid = 0;  // launches by cudaLaunchKernelEx, the last one's CTAs
 
 extern "C" {
@@ -32,7 +34,10 @@ cudaError_t cudaEventElapsedTime(float *t, cudaEvent_t, cudaEvent_t) { return *t
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaMalloc(void **p, size_t n) { return (*p = std::calloc(n + 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
-cudaError_t cudaMallocHost(void **p, size_t n) { return cudaMalloc(p, n); }
+cudaError_t cudaMallocHost(void **p, size_t n) {
+  ++n_pinned;
+  return fail_pinned ? cudaErrorMemoryAllocation : cudaMalloc(p, n);
+}
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
 cudaError_t cudaFree(void *p) { return std::free(p), cudaSuccess; }
 cudaError_t cudaFreeHost(void *p) { return cudaFree(p); }
@@ -78,7 +83,18 @@ unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, cudaStream_t) { return 
 cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *) { return *k = nullptr, cudaSuccess; }
 cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **, size_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return *s = nullptr, cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { return ++n_streams, *s = nullptr, cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaMemset(void *d, int v, size_t n) { return std::memset(d, v, n), cudaSuccess; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes *a, const void *p) {
+  a->type = p == page_locked ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
+  return cudaSuccess;
+}
+static int encoded(void) { return 0; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *, void **p, unsigned, unsigned long long, cudaDriverEntryPointQueryResult *q) {
+  *p = (void *)encoded;
+  return *q = cudaDriverEntryPointSuccess, cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 }  // extern "C"

@@ -37,14 +37,23 @@ def exe(tmp_path_factory):
                   (os.path.join(here, "solver_host.cpp"), "cu"), (os.path.join(csrc, "pdlp_capi.cu"), ""))
 
 
-@pytest.fixture(scope="module")
-def batch_exe(tmp_path_factory):
+def _with_library_object(out, driver, obj):
     from paper_2311_12180_gb300 import _build as B
 
     B.build()
     here = os.path.join(ROOT, "tests")
-    return _build(str(tmp_path_factory.mktemp("batch") / "batch_host"), (os.path.join(here, "cuda_runtime_host.cpp"), ""),
-                  (os.path.join(here, "batch_host.cpp"), "cu"), (os.path.join(B.OBJDIR, "pdlp_batch.cu.o"), ""))
+    return _build(str(out / "host"), (os.path.join(here, "cuda_runtime_host.cpp"), ""), (os.path.join(here, driver), "cu"),
+                  (os.path.join(B.OBJDIR, obj), ""))
+
+
+@pytest.fixture(scope="module")
+def batch_exe(tmp_path_factory):
+    return _with_library_object(tmp_path_factory.mktemp("batch"), "batch_host.cpp", "pdlp_batch.cu.o")
+
+
+@pytest.fixture(scope="module")
+def mlp_exe(tmp_path_factory):
+    return _with_library_object(tmp_path_factory.mktemp("mlp"), "mlp_host.cpp", "pdlp_mlp.cu.o")
 
 
 def _run(exe, *args):
@@ -101,3 +110,16 @@ def test_a_batch_fits_its_grid_to_the_stream(batch_exe, resident, small, large):
         assert resident / 4 < create[2]["grid"] <= resident or create[2]["grid"] == 4 <= resident
     else:
         assert create[2]["grid"] == 152
+
+
+def test_page_locked_chunks_come_with_the_first_large_pageable_prediction(mlp_exe):
+    create, small, locked, large, batches = _run(mlp_exe, 0)
+    assert all(r[1] == P.OK and r[2]["written"] for r in (create, small, locked, large, batches))
+    assert [r[2]["pinned"] for r in (create, small, locked, large, batches)] == [0, 0, 0, 1, 1]
+    assert [r[2]["streams"] for r in (create, small, locked, large, batches)] == [1, 1, 1, 9, 9]
+
+
+def test_predictions_without_page_locked_memory(mlp_exe):
+    rows = _run(mlp_exe, 1)
+    assert all(r[1] == P.OK and r[2]["written"] for r in rows)
+    assert rows[-1][2]["pinned"] == 1  # asked for once
