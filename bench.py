@@ -896,7 +896,7 @@ def main():
         cpu = cpu_baseline(lp)
 
     kernels_per_period = 2 * (period + max(4, period // 8)) + 4  # + check_primal, infeas, check_dual, restart
-    if lay["K_stored"] + lay["KT_stored"] + 8 * (lp.m + lp.n) <= 8_000_000:
+    if lay["period_ctas"]:
         kernels_per_period = 1  # a small LP's period is one launch
     line = {
         "metric": METRIC,

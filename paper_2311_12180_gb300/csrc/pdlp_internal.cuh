@@ -172,7 +172,12 @@ struct SolverState {
 };
 constexpr int PERIOD_CLUSTER = 16;
 constexpr int PERIOD_SHARE_MAX = 200 * 1024;
-constexpr int64_t PERIOD_WORK_MAX = 8000000;
+// the largest LPs that take it (see period_plan): stored entries, long rows,
+// and slices of K and K' with the matrix resident or not; long rows on one
+// cluster; stored entries and slices with FP32 values
+constexpr int64_t PERIOD_STORED_MAX = 4500000, PERIOD_STORED_F32_MAX = 900000;
+constexpr int PERIOD_LONG_MAX = 14000, PERIOD_SLICES_MAX = 17000, PERIOD_SLICES_L2_MAX = 12000;
+constexpr int PERIOD_LONG_CLUSTER_MAX = 350, PERIOD_SLICES_F32_MAX = 4000;
 constexpr int PERIOD_PART_GROUPS = 4096;  // partial sums of each value: groups, or a cluster's virtual warps
 // The grids (256-thread CTAs) of the kernels whose sums a period reproduces.
 struct PeriodGrids {

@@ -24,10 +24,10 @@
 //   * The check's phases are out of line, and little that the steps use lives
 //     in local memory: each barrier's acquire empties the L1, so a spilled
 //     register costs an L2 round trip.
-// Measured per iteration, step and check kernels against this one: 18.4 / 8.2
-// us on a 200 x 500 LP, 20.3 / 14.7 on the 200 x 300 transportation LP, 23.4 /
-// 14.9 at 1e5 nonzeros of the power-law recipe, 36.4 / 29.9 at 1e6, 44.1 /
-// 40.8 at 2e6.  From 1e6 on the FP64 pipe bounds it (each row's epilogue and
+// Measured per iteration of a long run, step and check kernels against this
+// one: 16.9 / 8.2 us on a 200 x 500 LP, 18.5 / 15.5 on the 200 x 300
+// transportation LP, 21.5 / 14.8 at 1e5 nonzeros of the power-law recipe, 35.5 /
+// 29.9 at 1e6, 42.5 / 40.2 at 2e6.  From 1e6 on the FP64 pipe bounds it (each row's epilogue and
 // each virtual warp's sums take whole warp instructions), and the gathers in
 // flight: half of the step kernels' warps are gone.
 //
@@ -867,17 +867,37 @@ void launch_config(const PeriodPlan &p, cudaStream_t s, cudaLaunchConfig_t &cfg,
 // share a GPC), the step and check kernels run the LP; too few SMs for the
 // whole-GPU kernel show at its cooperative launch.
 //
-// LPs above PERIOD_WORK_MAX (stored entries of K and K' plus eight per row and
-// column) keep the step and check kernels: 6.4e6 at 2e6 nonzeros of the
-// power-law recipe, where this path takes 0.93 of their time; at 3e6 (9.6e6)
-// an earlier build without resident shares took 1.03.
+// Larger LPs keep the step and check kernels, whose grids have twice the warps:
+// with many items, this path's warps walk them one after another.  Where the
+// lines lie, in us an iteration, step kernels / this path:
+//   stored entries  power-law recipe, 1e6 nonzeros 36 / 30 (2.0e6 stored), 2e6
+//                   42.5 / 40.2 (4.07e6), 2.2e6 42.3 / 42.1 (4.47e6), 2.3e6
+//                   43.8 / 45.0 (4.68e6), 3e6 48.5 / 67
+//   long rows       rows of 60 entries in K and K': 7000 of each 29.7 / 27.8,
+//                   10000 of each 31.8 / 36.4, 30000 of each 47 / 66
+//   slices          transportation, 600 x 900 (16900, resident) 37.0 / 31.5,
+//                   600 x 1000 (18800, not resident) 38.0 / 40.3; not resident:
+//                   power law 1.8e5 x 1.8e5 (11100) 46.9 / 44.5, 3e5 x 1e5 of 4
+//                   a row (12500) 34.7 / 38.7
+//   long rows on one cluster, whose few warps pay each row's own sums: 300 in all
+//                   (150 x 150 of 80) 15.9 / 13.6, 400 15.0 (whole GPU 13.5),
+//                   600 19.5 (11.5)
+//   FP32 values     the whole-GPU kernel of this mode also holds the FP64 product
+//                   and spills: 2e5 nonzeros 21.6 / 19.3, 5e5 24.0 / 24.1, 1e6
+//                   34.2 / 36.0; 60000 x 60000 of 4 a row (3750 slices) 18.9 /
+//                   18.3, 1e5 x 1e5 of 3 (6250) 21.8 / 23.0
 void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int nk, const int4 *t_items, int nt,
                  int64_t stored, int value_bytes, int num_sms, cudaStream_t s) {
-  if (stored + 8 * ((int64_t)m + n) > PERIOD_WORK_MAX) return;
+  int slices = 0;
+  for (int i = 0; i < nk; ++i) slices += k_items[i].y > 0;
+  for (int i = 0; i < nt; ++i) slices += t_items[i].y > 0;
+  const int longs = nk + nt - slices;
+  if (stored > PERIOD_STORED_MAX || longs > PERIOD_LONG_MAX || slices > PERIOD_SLICES_MAX) return;
   const PeriodGrids &g = p.grids;
   const double f64 = (double)stored / 32 + 6.0 * n / 32 + 9.0 * m / 32;
   const double extra = 19.0 * f64 * (1.0 / PERIOD_CLUSTER - 1.0 / num_sms);
-  p.cluster = extra < 2.0 * 1900.0;
+  p.cluster = extra < 2.0 * 1900.0 && longs <= PERIOD_LONG_CLUSTER_MAX;
+  if (!p.cluster && value_bytes == 4 && (stored > PERIOD_STORED_F32_MAX || slices > PERIOD_SLICES_F32_MAX)) return;
   p.ctas = p.cluster ? PERIOD_CLUSTER : num_sms;
   const int most_groups = std::max({g.primal, g.dual, g.check_primal, g.check_dual, g.infeas, g.restart});
   if (most_groups > (p.cluster ? PERIOD_PART_GROUPS / 8 : MAX_SLOTS * num_sms)) {
@@ -899,6 +919,10 @@ void period_plan(PeriodPlan &p, int32_t m, int32_t n, const int4 *k_items, int n
   deal(t_items, nt, g.primal);
   const int64_t most = *std::max_element(bytes.begin(), bytes.end());
   p.share_bytes = most <= PERIOD_SHARE_MAX ? (int)((most + 1023) / 1024 * 1024) : 0;
+  if (!p.share_bytes && slices > PERIOD_SLICES_L2_MAX) {
+    p.ctas = 0;
+    return;
+  }
   if (p.cluster) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at[1];
