@@ -588,9 +588,10 @@ int create_common(pdlp_solver **out, int32_t m, int32_t n, int32_t n_eq, const d
     cudaError_t e;
     if (have_perm) {
       const int32_t *perm = twork + wcs + n, *rowid = perm + nnz;
-      // reciprocal scratch: the x_last / y_last slots, unused until a solve begins
+      // scratch for reciprocals and lists: vectors that a solve writes before it reads them
       e = setup_scale_perm(m, n, nnz, s->K_ptr, s->K_idx, s->K_val, s->T_ptr, s->T_val, rowid, perm, s->D1, s->D2,
-                           s->work_m, s->work_n, VM(9), VN(12), prm.ruiz_iters, prm.pc_alpha, st);
+                           s->work_m, s->work_n, VM(9), VN(12), (int32_t *)VM(8), (int32_t *)VN(11), prm.ruiz_iters,
+                           prm.pc_alpha, st);
     } else {
       // norms, reciprocals and lists in vectors that a solve writes before it reads them
       const ScaleWork w{VM(11), VN(14), s->work_m, s->work_n, VM(9), VN(12), (int32_t *)VM(8), (int32_t *)VN(11)};

@@ -30,11 +30,13 @@ __device__ __forceinline__ double warp_add(double v) {
 }
 
 // Rows of more than LONG_ROW entries are taken by a warp each, whichever they
-// lie next to; k_long_rows lists them (list[0..), their number in list[rows],
-// zeroed before; the order is of no account).  48: at 96, 1000 rows of 100 take
+// lie next to; k_long_rows lists those of K and of K' (list[0..), their number
+// in list[rows], zeroed by k_unit; the order is of no account).  Where the GPU has a warp for
+// every row, all of them are, without a list.  48: at 96, 1000 rows of 100 take
 // 591 us instead of 289, at 32 30000 rows of 100 take 1733 instead of 1564.
 constexpr int LONG_ROW = 48;
-__global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t rows, int32_t *__restrict__ list) {
+__device__ __forceinline__ void list_long_rows(const int32_t *__restrict__ ptr, int32_t rows,
+                                               int32_t *__restrict__ list) {
   const int lane = threadIdx.x & 31;
   for (long long r0 = (long long)blockIdx.x * ST + threadIdx.x - lane; r0 < rows; r0 += (long long)gridDim.x * ST) {
     const long long r = r0 + lane;
@@ -44,6 +46,22 @@ __global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t rows, int32
     if (lane == 0 && all) at = atomicAdd(list + rows, __popc(all));
     at = __shfl_sync(0xffffffffu, at, 0) + __popc(all & ((1u << lane) - 1u));
     if (is) list[at] = (int32_t)r;
+  }
+}
+__global__ void k_long_rows(const int32_t *K_ptr, int32_t m, int32_t *long_m, const int32_t *T_ptr, int32_t n,
+                            int32_t *long_n) {
+  if (long_m) list_long_rows(K_ptr, m, long_m);
+  if (long_n) list_long_rows(T_ptr, n, long_n);
+}
+
+// D1 = 1, D2 = 1, and empty lists of long rows (null: none).
+__global__ void k_unit(int32_t m, int32_t n, double *__restrict__ D1, double *__restrict__ D2, int32_t *long_m,
+                       int32_t *long_n) {
+  for (long long k = (long long)blockIdx.x * ST + threadIdx.x; k < (long long)m + n; k += (long long)gridDim.x * ST)
+    (k < m ? D1[k] : D2[k - m]) = 1.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (long_m) long_m[m] = 0;
+    if (long_n) long_n[n] = 0;
   }
 }
 
@@ -141,9 +159,9 @@ __global__ void __launch_bounds__(ST, SCALE_CTAS) k_scale_rows(const int32_t *__
     const unsigned long long bits = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
     return bits > 0x7ff0000000000000ull ? 0ull : bits;
   };
-  const int32_t count = longs[rows];
+  const int32_t count = longs ? longs[rows] : rows;
   for (long long i = warp; i < count; i += nwarps) {
-    const int32_t row = longs[i];
+    const int32_t row = longs ? longs[i] : (int32_t)i;
     const unsigned b = ptr[row], end = ptr[row + 1];
     const double fa = SCALE ? (KMAJOR ? r : s)[row] : 1.0, fr = SCALE ? (KMAJOR ? rr : rs)[row] : 1.0;
     unsigned long long most = 0;
@@ -181,6 +199,7 @@ __global__ void __launch_bounds__(ST, SCALE_CTAS) k_scale_rows(const int32_t *__
       if (lane == 0) maxima[row] = most;
     }
   }
+  if (!longs) return;
   for (long long r0 = warp * SCALE_ROWS; r0 < rows; r0 += nwarps * SCALE_ROWS) {
     // starts of the warp's rows (lanes 0..SCALE_ROWS - 1) and the end of the last
     const int start = lane <= SCALE_ROWS ? ptr[min((long long)rows, r0 + lane)] : 0;
@@ -313,10 +332,6 @@ __global__ void k_copy_perm(const int32_t *__restrict__ perm, const double *__re
     tval[p] = kval[perm[p]];
 }
 
-__global__ void k_fill(double *__restrict__ a, int32_t n, double v) {
-  for (int i = blockIdx.x * ST + threadIdx.x; i < n; i += gridDim.x * ST) a[i] = v;
-}
-
 __global__ void k_vectors(int32_t m, int32_t n, const double *__restrict__ c0, const double *__restrict__ q0,
                           const double *__restrict__ l0, const double *__restrict__ u0, const double *__restrict__ D1,
                           const double *__restrict__ D2, double *__restrict__ c, double *__restrict__ q,
@@ -432,17 +447,20 @@ constexpr int FULL_WARPS = 152 * 64;
 int scale_grid(long long rows) {
   return std::max(grid_for(rows * 32 / SCALE_ROWS), std::min(grid_for(32 * rows), FULL_WARPS * 32 / ST));
 }
-// The list of long rows (rows + 1 ints).
-cudaError_t long_rows(const int32_t *ptr, int32_t rows, int32_t *list, cudaStream_t s) {
-  const cudaError_t e = cudaMemsetAsync(list + rows, 0, sizeof(int32_t), s);
-  if (e == cudaSuccess) k_long_rows<<<grid_for(rows), ST, 0, s>>>(ptr, rows, list);
-  return e;
+// D1 = D2 = 1, and the lists of long rows of K and K' into lm and ln (m + 1 and
+// n + 1 ints); null, and no list, where the rows have a warp each.
+void unit_and_lists(int32_t m, int32_t n, const int32_t *K_ptr, const int32_t *T_ptr, double *D1, double *D2,
+                    int32_t *&lm, int32_t *&ln, cudaStream_t s) {
+  if (m <= FULL_WARPS) lm = nullptr;
+  if (n <= FULL_WARPS) ln = nullptr;
+  k_unit<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, D1, D2, lm, ln);
+  if (lm || ln) k_long_rows<<<grid_for(std::max(lm ? m : 0, ln ? n : 0)), ST, 0, s>>>(K_ptr, m, lm, T_ptr, n, ln);
 }
-// Row sums: a row a warp while the GPU has the warps (`longs` unused), else 32
+// Row sums: a row a warp while the GPU has the warps (`longs` null), else 32
 // and the long ones by themselves.
 void row_sums(const int32_t *ptr, const double *val, int32_t rows, const int32_t *longs, double *out, double p,
               cudaStream_t s) {
-  if (rows <= FULL_WARPS)
+  if (!longs)
     k_row_sum<<<grid_for(32LL * rows), ST, 0, s>>>(ptr, val, rows, 1, nullptr, out, p);
   else
     k_row_sum<<<std::max(grid_for(rows), FULL_WARPS * 32 / ST), ST, 0, s>>>(ptr, val, rows, 32, longs, out, p);
@@ -454,31 +472,28 @@ cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32
                         int32_t *T_ptr, int32_t *T_idx, double *T_val, double *D1, double *D2, const ScaleWork &w,
                         int ruiz_iters, double pc_alpha, cudaStream_t s) {
   (void)nnz;
-  if (m > 0) k_fill<<<grid_for(m), ST, 0, s>>>(D1, m, 1.0);
-  k_fill<<<grid_for(n), ST, 0, s>>>(D2, n, 1.0);
+  int32_t *lm = w.long_m, *ln = w.long_n;
+  unit_and_lists(m, n, K_ptr, T_ptr, D1, D2, lm, ln, s);
   unsigned long long *const mm = reinterpret_cast<unsigned long long *>(w.norm_m),
                            *const mn = reinterpret_cast<unsigned long long *>(w.norm_n);
-  cudaError_t e = m > 0 ? long_rows(K_ptr, m, w.long_m, s) : cudaSuccess;
-  if (e == cudaSuccess) e = long_rows(T_ptr, n, w.long_n, s);
-  if (e != cudaSuccess) return e;
   const int gm = scale_grid(m), gn = scale_grid(n);
   if (ruiz_iters > 0) {  // the first pass's maxima
     if (m > 0)
-      k_scale_rows<false, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.long_m, nullptr, nullptr, nullptr, nullptr, mm);
-    k_scale_rows<false, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.long_n, nullptr, nullptr, nullptr, nullptr, mn);
+      k_scale_rows<false, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, lm, nullptr, nullptr, nullptr, nullptr, mm);
+    k_scale_rows<false, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, ln, nullptr, nullptr, nullptr, nullptr, mn);
   }
   const int passes = ruiz_iters + (pc_alpha >= 0.0 ? 1 : 0);
   for (int it = 0; it < passes; ++it) {
     if (it >= ruiz_iters) {  // Pock-Chambolle: row sums of K and K'
-      if (m > 0) row_sums(K_ptr, K_val, m, w.long_m, w.norm_m, 2.0 - pc_alpha, s);
-      row_sums(T_ptr, T_val, n, w.long_n, w.norm_n, pc_alpha, s);
+      if (m > 0) row_sums(K_ptr, K_val, m, lm, w.norm_m, 2.0 - pc_alpha, s);
+      row_sums(T_ptr, T_val, n, ln, w.norm_n, pc_alpha, s);
     }
     k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, w.norm_m, w.norm_n, w.f_m, w.f_n, w.rcp_m, w.rcp_n, D1, D2);
     const bool more = it + 1 < ruiz_iters;  // the next pass needs maxima
     if (m > 0)
-      k_scale_rows<true, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, w.long_m, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+      k_scale_rows<true, true><<<gm, ST, 0, s>>>(K_ptr, K_idx, K_val, m, lm, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
                                                  more ? mm : nullptr);
-    k_scale_rows<true, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, w.long_n, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
+    k_scale_rows<true, false><<<gn, ST, 0, s>>>(T_ptr, T_idx, T_val, n, ln, w.f_m, w.rcp_m, w.f_n, w.rcp_n,
                                                 more ? mn : nullptr);
   }
   return cudaGetLastError();
@@ -487,9 +502,9 @@ cudaError_t setup_scale(int32_t m, int32_t n, int64_t nnz, int32_t *K_ptr, int32
 cudaError_t setup_scale_perm(int32_t m, int32_t n, int64_t nnz, const int32_t *K_ptr, const int32_t *K_idx,
                              double *K_val, const int32_t *T_ptr, double *T_val, const int32_t *rowid,
                              const int32_t *perm, double *D1, double *D2, double *work_m, double *work_n,
-                             double *rcp_m, double *rcp_n, int ruiz_iters, double pc_alpha, cudaStream_t s) {
-  if (m > 0) k_fill<<<grid_for(m), ST, 0, s>>>(D1, m, 1.0);
-  k_fill<<<grid_for(n), ST, 0, s>>>(D2, n, 1.0);
+                             double *rcp_m, double *rcp_n, int32_t *long_m, int32_t *long_n, int ruiz_iters,
+                             double pc_alpha, cudaStream_t s) {
+  unit_and_lists(m, n, K_ptr, T_ptr, D1, D2, long_m, long_n, s);
   const int eg = grid_for(nnz);
   for (int it = 0; it < ruiz_iters; ++it) {
     cudaError_t e = cudaMemsetAsync(work_m, 0, sizeof(double) * (size_t)m, s);
@@ -503,13 +518,8 @@ cudaError_t setup_scale_perm(int32_t m, int32_t n, int64_t nnz, const int32_t *K
   }
   if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);
   if (pc_alpha >= 0.0) {  // Pock-Chambolle: row sums over K, column sums over K' (fixed order)
-    // the lists of long rows in the reciprocals' place, which k_factors writes after
-    int32_t *const lm = reinterpret_cast<int32_t *>(rcp_m), *const ln = reinterpret_cast<int32_t *>(rcp_n);
-    cudaError_t e = m > FULL_WARPS ? long_rows(K_ptr, m, lm, s) : cudaSuccess;
-    if (e == cudaSuccess && n > FULL_WARPS) e = long_rows(T_ptr, n, ln, s);
-    if (e != cudaSuccess) return e;
-    if (m > 0) row_sums(K_ptr, K_val, m, lm, work_m, 2.0 - pc_alpha, s);
-    row_sums(T_ptr, T_val, n, ln, work_n, pc_alpha, s);
+    if (m > 0) row_sums(K_ptr, K_val, m, long_m, work_m, 2.0 - pc_alpha, s);
+    row_sums(T_ptr, T_val, n, long_n, work_n, pc_alpha, s);
     k_factors<<<grid_for((long long)m + n), ST, 0, s>>>(m, n, work_m, work_n, work_m, work_n, rcp_m, rcp_n, D1, D2);
     if (nnz > 0) k_scale_entries<<<eg, ST, 0, s>>>(K_idx, rowid, K_val, nnz, work_m, work_n, rcp_m, rcp_n);
     if (nnz > 0) k_copy_perm<<<eg, ST, 0, s>>>(perm, K_val, nnz, T_val);

@@ -54,7 +54,7 @@ cudaError_t setup_scale(int32_t, int32_t, int64_t, int32_t *, int32_t *, double 
                         double *, const ScaleWork &, int, double, cudaStream_t) { return cudaSuccess; }
 cudaError_t setup_scale_perm(int32_t, int32_t, int64_t, const int32_t *, const int32_t *, double *, const int32_t *, double *,
                              const int32_t *, const int32_t *, double *, double *, double *, double *, double *, double *,
-                             int, double, cudaStream_t) { return cudaSuccess; }
+                             int32_t *, int32_t *, int, double, cudaStream_t) { return cudaSuccess; }
 cudaError_t setup_vectors(int32_t, int32_t, const double *, const double *, const double *, const double *, const double *,
                           const double *, double *, double *, double *, double *, cudaStream_t) { return cudaSuccess; }
 cudaError_t setup_f32(int64_t, const double *, float *, cudaStream_t) { return cudaSuccess; }
