@@ -670,11 +670,12 @@ bool vec4(const float *p, int ld) { return reinterpret_cast<uintptr_t>(p) % 16 =
 
 // Copies of large results into the caller's pageable memory (copy_out).
 constexpr int COPY_THREADS = 8;
-constexpr size_t COPY_CHUNK = size_t(1) << 19, COPY_MIN = size_t(8) << 20;
+constexpr size_t COPY_CHUNK = size_t(1) << 19, COPY_MIN = size_t(8) << 20, COPY_ONCE = size_t(32) << 20;
 struct HostCopy {
   char *pinned = nullptr;  // two chunks a thread
   cudaStream_t st[COPY_THREADS] = {};
   cudaEvent_t ready = nullptr;
+  int seen = 0;  // results of COPY_MIN so far that went by a plain copy
   bool tried = false;
 };
 
@@ -764,12 +765,14 @@ cudaError_t copy_chunks(const HostCopy &hc, int device, int t, char *dst, const 
   return e != cudaSuccess ? e : d;
 }
 
-// The pinned chunks and streams of copy_out, made at a net's first large
-// prediction into pageable memory (0.4 ms; a net that only trains has none).
-// Without page-locked memory to be had its copies are plain ones.
-void host_copy_init(pdlp_mlp *M) {
+// The pinned chunks and streams of copy_out, made where they first pay for the
+// 0.4 ms that they take: at a net's first result of COPY_ONCE into pageable
+// memory (2 ms of faults saved at 121 MB) or its second of COPY_MIN; a net that
+// only trains has none.  Without page-locked memory to be had its copies are
+// plain ones.
+void host_copy_init(pdlp_mlp *M, size_t bytes) {
   HostCopy &hc = M->hc;
-  if (hc.tried) return;
+  if (hc.tried || (bytes < COPY_ONCE && !hc.seen++)) return;
   hc.tried = true;
   char *p = nullptr;
   cudaError_t e = cudaMallocHost((void **)&p, 2 * COPY_THREADS * COPY_CHUNK);
@@ -802,7 +805,7 @@ int copy_out(pdlp_mlp *M, float *dst, const float *src, size_t count) {
     staged = false;
   }
   staged = staged && pa.type == cudaMemoryTypeUnregistered;
-  if (staged) host_copy_init(M);
+  if (staged) host_copy_init(M, bytes);
   if (!staged || !hc.pinned) {
     MCK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, M->stream));
     return PDLP_OK;

@@ -40,8 +40,13 @@ int main(int argc, char **argv) {
   };
   predict("small", 20, false);
   predict("locked", 64, true);
-  predict("large", 64, false);
+  predict("first", 64, false);
+  predict("second", 64, false);
   predict("batches", 150, false);  // two staged ones and a small rest
+  pdlp_mlp_destroy(net);
+  // 36.8 MB a prediction: the first one pays
+  show("big", pdlp_mlp_create(&net, in, hid, out, 256, nullptr));
+  predict("once", 230, false);
   pdlp_mlp_destroy(net);
   return 0;
 }
