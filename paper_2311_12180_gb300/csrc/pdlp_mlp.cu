@@ -26,6 +26,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <cmath>
@@ -787,14 +789,30 @@ void host_copy_init(pdlp_mlp *M, size_t bytes) {
   }
 }
 
-// Device memory into the caller's, after what the stream holds.  A large
-// pageable destination is bound by the host's page faults: of 5.2 ms for a
-// fresh 121 MB one thread's faults are 3 to 4, the transfer itself is 0.64.
-// With the faults taken by the memcpys of several threads, a prediction of 500
-// x 60500 takes 3.7 ms instead of 5.4 (2.9 instead of 4.7 alone); mapping the
-// pages ahead by madvise on as many threads gave 5.1.  Below COPY_MIN (about
-// 0.3 ms of faults) the threads' start costs about what they save; page-locked
-// and managed destinations need no staging.
+// Whether the destination's pages are there already: sixteen of them, the first
+// and the last among them.  Memory that is not the process's is the plain
+// copy's to refuse.
+bool pages_present(const char *p, size_t bytes) {
+  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+  for (int i = 0; i < 16; ++i) {
+    const uintptr_t at = (uintptr_t)p + (bytes - 1) / 15 * i + (i == 15 ? (bytes - 1) % 15 : 0);
+    unsigned char in;
+    if (mincore((void *)(at / page * page), 1, &in) != 0) return true;
+    if (!(in & 1)) return false;
+  }
+  return true;
+}
+
+// Device memory into the caller's, after what the stream holds.  A large fresh
+// pageable destination is bound by the host's page faults: of 5.2 ms for 121 MB
+// one thread's faults are 3 to 4, the transfer itself is 0.64.  With the faults
+// taken by the memcpys of several threads, a prediction of 500 x 60500 into
+// fresh memory takes 2.8 ms instead of 5.1 (into half-written memory 2.6 instead
+// of 40); mapping the pages ahead by madvise on as many threads gained little.
+// Where the pages are there, the plain copy is the faster one: 0.97 ms against
+// 2.4, and 0.2 against 0.55 for 13 MB.  Below COPY_MIN (about 0.3 ms of faults)
+// the threads' start costs about what they save; page-locked and managed
+// destinations need no staging.
 int copy_out(pdlp_mlp *M, float *dst, const float *src, size_t count) {
   const size_t bytes = sizeof(float) * count;
   cudaPointerAttributes pa{};
@@ -804,7 +822,7 @@ int copy_out(pdlp_mlp *M, float *dst, const float *src, size_t count) {
     cudaGetLastError();
     staged = false;
   }
-  staged = staged && pa.type == cudaMemoryTypeUnregistered;
+  staged = staged && pa.type == cudaMemoryTypeUnregistered && !pages_present((const char *)dst, bytes);
   if (staged) host_copy_init(M, bytes);
   if (!staged || !hc.pinned) {
     MCK(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, M->stream));

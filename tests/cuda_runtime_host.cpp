@@ -12,6 +12,7 @@ int fail_capture = 0;          // cudaStreamEndCapture fails
 int capturing = 0, n_graph = 0;  // between begin and end of a capture; graph launches
 int resident_ctas = 1 << 30;     // a cooperative launch of more is refused
 int n_pinned = 0, n_streams = 0, fail_pinned = 0;  // calls of cudaMallocHost and cudaStreamCreateWithFlags
+int device_fill = 0;                               // every byte of new device memory
 const void *page_locked = nullptr;                 // this address is page-locked memory, all others are pageable
 int n_launch = 0, last_grid = 0;  // launches by cudaLaunchKernelEx, the last one's CTAs
 
@@ -33,7 +34,11 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *t, cudaEvent_t, cudaEvent_t) { return *t = 0.f, cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaMalloc(void **p, size_t n) { return (*p = std::calloc(n + 1, 1)) ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMalloc(void **p, size_t n) {
+  if (!(*p = std::malloc(n + 1))) return cudaErrorMemoryAllocation;
+  std::memset(*p, device_fill, n + 1);
+  return cudaSuccess;
+}
 cudaError_t cudaMallocHost(void **p, size_t n) {
   ++n_pinned;
   return fail_pinned ? cudaErrorMemoryAllocation : cudaMalloc(p, n);

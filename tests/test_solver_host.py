@@ -116,11 +116,11 @@ def test_page_locked_chunks_come_where_a_large_pageable_prediction_pays_for_them
     rows = _run(mlp_exe, 0)
     assert all(r[1] == P.OK and r[2]["written"] for r in rows)
     assert [(r[0], r[2]["pinned"], r[2]["streams"]) for r in rows] == [
-        ("create", 0, 1), ("small", 0, 1), ("locked", 0, 1), ("first", 0, 1), ("second", 1, 9), ("batches", 1, 9),
-        ("big", 1, 10), ("once", 2, 18)]
+        ("create", 0, 1), ("small", 0, 1), ("locked", 0, 1), ("written", 0, 1), ("first", 0, 1), ("second", 1, 9),
+        ("batches", 1, 9), ("big", 1, 10), ("written", 1, 10), ("once", 2, 18)]
 
 
 def test_predictions_without_page_locked_memory(mlp_exe):
     rows = _run(mlp_exe, 1)
     assert all(r[1] == P.OK and r[2]["written"] for r in rows)
-    assert [r[2]["pinned"] for r in rows] == [0, 0, 0, 0, 1, 1, 1, 2]  # asked for once a network
+    assert [r[2]["pinned"] for r in rows] == [0, 0, 0, 0, 0, 1, 1, 1, 1, 2]  # asked for once a network
