@@ -258,8 +258,14 @@ void mark_in_flight(pdlp_solver *s, bool on) {
 // stream has too few SMs for CTAs that wait on one another (a green context's
 // or an MPS client's share; nothing has run), the solver goes over to the step
 // and check kernels for good: the same bits, on any number of SMs.
+// A stream under capture is refused, as the launch of the graph is there: the
+// work would be recorded, not done.
 int try_period(pdlp_solver *s, int max_trials, bool *done) {
   *done = false;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(s->stream, &capture));
+  if (capture != cudaStreamCaptureStatusNone)
+    return fail(PDLP_ERR_CUDA, "a check period cannot be enqueued on a stream under capture");
   mark_in_flight(s, true);
   if (!s->period.ctas || (!s->period.cluster && g_in_flight[s->device % 64] > 1)) return PDLP_OK;
   const cudaError_t e = launch_period(s->period, s->K, s->KT, s->V, s->st, max_trials, s->stream);

@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 
+int stream_captured = 0;        // the caller captures the solver's stream
 int fail_capture = 0;          // cudaStreamEndCapture fails
 int capturing = 0, n_graph = 0;  // between begin and end of a capture; graph launches
 int resident_ctas = 1 << 30;     // a cooperative launch of more is refused
@@ -64,6 +65,9 @@ cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned long 
   return *x = (cudaGraphExec_t)(size_t)1, cudaSuccess;
 }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t) { return x ? (++n_graph, cudaSuccess) : cudaErrorInvalidValue; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *c) {
+  return *c = stream_captured ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone, cudaSuccess;
+}
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return capturing = 1, cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
   capturing = 0;

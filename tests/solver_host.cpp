@@ -12,7 +12,7 @@
 #include "pdlp_internal.cuh"
 #include "pdlp_setup.cuh"
 
-extern int fail_capture, capturing, n_graph;     // of the runtime's stand-in
+extern int fail_capture, capturing, n_graph, stream_captured;     // of the runtime's stand-in
 static int plan_ctas = 0;                        // what period_plan decides
 static bool plan_cluster = false;
 static cudaError_t period_error = cudaSuccess;   // of launch_period
@@ -115,6 +115,17 @@ int main(int argc, char **argv) {
     pdlp_layout_info info;
     show("layout", pdlp_get_layout(s, &info));
     show("ctas", info.period_ctas);
+    pdlp_destroy(s);
+    return 0;
+  }
+  if (scenario == "captured" || scenario == "captured graph") {  // the caller captures the solver's stream
+    plan_ctas = scenario == "captured" ? 152 : 0;
+    pdlp_solver *s = create();
+    show("begin", pdlp_begin(s, nullptr, nullptr, 1e-6, 100));
+    stream_captured = 1;
+    show("run", pdlp_run_periods(s, 2));
+    stream_captured = 0;
+    show("run", pdlp_run_periods(s, 2));
     pdlp_destroy(s);
     return 0;
   }

@@ -124,3 +124,11 @@ def test_predictions_without_page_locked_memory(mlp_exe):
     rows = _run(mlp_exe, 1)
     assert all(r[1] == P.OK and r[2]["written"] for r in rows)
     assert [r[2]["pinned"] for r in rows] == [0, 0, 0, 0, 0, 1, 1, 1, 1, 2]  # asked for once a network
+
+
+@pytest.mark.parametrize("scenario", ["captured", "captured graph"])
+def test_periods_are_refused_on_a_stream_under_capture(exe, scenario):
+    begin, refused, run = _run(exe, scenario)
+    assert begin[1] == P.OK and refused[1] == P.ERR_CUDA and run[1] == P.OK
+    kind = "period" if scenario == "captured" else "graph"
+    assert refused[2][kind] == begin[2][kind] and run[2][kind] == begin[2][kind] + 2
