@@ -60,9 +60,24 @@ struct Layout {
   }
 };
 
+// Solvers of each device that have work enqueued which the host has not yet
+// waited for, and batched solves and network calls under way
+// (count_in_flight).  A whole-GPU period holds every SM, so solvers on several streams
+// would take turns, where the step kernels of small LPs share the GPU: four LPs
+// of 1e5 nonzeros take 7.9 us an iteration each as step kernels and 14.7 as
+// whole-GPU periods (alone 29.7 and 15.1), sixteen 3.1 and 14.8; two of 1e6
+// 23.7 and 30.2; and a batch on some of the SMs would keep it waiting to the
+// batch's end.  So such a period runs while its solver is the only one; its
+// results are the step kernels' bits, whichever run.  (A cluster leaves room
+// for eight others: sixteen solvers of 2e4 nonzeros take 1.6 us, 2.7 as step
+// kernels.)
+std::atomic<int> g_in_flight[64];
+
 }  // namespace
 
 int pdlp::set_error(int code, const char *msg) { return fail(code, msg ? msg : ""); }
+
+void pdlp::count_in_flight(int device, int by) { g_in_flight[device % 64] += by; }
 
 struct pdlp_solver {
   int32_t m = 0, n = 0, n_eq = 0;
@@ -238,19 +253,8 @@ int build_graph(pdlp_solver *s) {
   return PDLP_OK;
 }
 
-// Solvers of each device that have work enqueued which the host has not yet
-// waited for.  A whole-GPU period holds every SM, so solvers on several streams
-// would take turns, where the step kernels of small LPs share the GPU: four LPs
-// of 1e5 nonzeros take 7.9 us an iteration each as step kernels and 14.7 as
-// whole-GPU periods (alone 29.7 and 15.1), sixteen 3.1 and 14.8; two of 1e6
-// 23.7 and 30.2.  So such a period runs while its solver is the only one; its
-// results are the step kernels' bits, whichever run.  (A cluster leaves room
-// for eight others: sixteen solvers of 2e4 nonzeros take 1.6 us, 2.7 as step
-// kernels.)
-std::atomic<int> g_in_flight[64];
-
 void mark_in_flight(pdlp_solver *s, bool on) {
-  if (s->in_flight != on) g_in_flight[s->device % 64] += on ? 1 : -1;
+  if (s->in_flight != on) count_in_flight(s->device, on ? 1 : -1);
   s->in_flight = on;
 }
 

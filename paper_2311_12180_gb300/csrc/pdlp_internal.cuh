@@ -205,6 +205,17 @@ cudaError_t kernels_init();  // one-time kernel attributes
 // Records `msg` as the calling thread's pdlp_last_error() and returns `code`.
 int set_error(int code, const char *msg);
 
+// Work on a device that whole-GPU periods should not wait for or hold up
+// (pdlp_capi.cu): one more or one less.
+void count_in_flight(int device, int by);
+struct InFlight {
+  int device;
+  explicit InFlight(int d) : device(d) { count_in_flight(device, 1); }
+  ~InFlight() { count_in_flight(device, -1); }
+  InFlight(const InFlight &) = delete;
+  InFlight &operator=(const InFlight &) = delete;
+};
+
 // Order-preserving integer key of an IEEE double (sign-magnitude -> two's
 // complement): a < b  <=>  key(a) < key(b) for non-NaN values (with -0 < +0).
 __device__ __forceinline__ long long dkey(double v) {

@@ -1131,6 +1131,7 @@ int pdlp_mlp_train(pdlp_mlp *M, int32_t steps, int32_t batch, const int32_t *idx
   for (long long i = 0; i < (long long)steps * batch; ++i)
     if (idx[i] < 0 || idx[i] >= M->samples) return set_error(PDLP_ERR_INVALID, "pdlp_mlp_train: index out of range");
   MCK(cudaSetDevice(M->device));
+  const pdlp::InFlight busy(M->device);
   int rc = ensure_idx(M, (size_t)steps * batch);
   if (rc) return rc;
   float *dloss = nullptr;
@@ -1160,6 +1161,7 @@ int pdlp_mlp_train(pdlp_mlp *M, int32_t steps, int32_t batch, const int32_t *idx
 int pdlp_mlp_predict(pdlp_mlp *M, int32_t count, const float *X, float *Y) {
   if (!M || count < 1 || !X || !Y) return set_error(PDLP_ERR_INVALID, "pdlp_mlp_predict: null argument or count < 1");
   MCK(cudaSetDevice(M->device));
+  const pdlp::InFlight busy(M->device);
   cudaStream_t s = M->stream;
   for (int b0 = 0; b0 < count; b0 += M->maxb) {
     const int B = std::min(M->maxb, count - b0);
@@ -1189,6 +1191,7 @@ int pdlp_mlp_gradients(pdlp_mlp *M, int32_t batch, const int32_t *idx, float *lo
   for (int i = 0; i < batch; ++i)
     if (idx[i] < 0 || idx[i] >= M->samples) return set_error(PDLP_ERR_INVALID, "pdlp_mlp_gradients: index out of range");
   MCK(cudaSetDevice(M->device));
+  const pdlp::InFlight busy(M->device);
   int rc = ensure_idx(M, batch);
   if (rc) return rc;
   cudaStream_t s = M->stream;

@@ -12,7 +12,12 @@
 
 extern int resident_ctas, last_grid;
 
+static int in_flight = 0, most_in_flight = 0;
 namespace pdlp {
+void count_in_flight(int, int by) {
+  in_flight += by;
+  if (in_flight > most_in_flight) most_in_flight = in_flight;
+}
 cudaError_t setup_pow_table(double *, long long, cudaStream_t) { return cudaSuccess; }
 int set_error(int code, const char *msg) {
   std::printf("error %d %s\n", code, msg);
@@ -46,9 +51,10 @@ int main(int argc, char **argv) {
   }
   pdlp_batch *b = nullptr;
   std::printf("create %d", pdlp_batch_create(&b, small + large, lps.data(), nullptr, nullptr));
-  std::printf(" grid %d\n", last_grid);
+  std::printf(" grid %d in_flight %d left %d\n", last_grid, most_in_flight, in_flight);
+  most_in_flight = 0;
   std::printf("solve %d", pdlp_batch_solve(b, nullptr, nullptr, 1e-6, 100, nullptr, nullptr, nullptr, nullptr));
-  std::printf(" grid %d\n", last_grid);
+  std::printf(" grid %d in_flight %d left %d\n", last_grid, most_in_flight, in_flight);
   pdlp_batch_destroy(b);
   return 0;
 }

@@ -15,7 +15,12 @@
 extern int n_pinned, n_streams, fail_pinned, device_fill;
 extern const void *page_locked;
 
+static int in_flight = 0, most_in_flight = 0;
 namespace pdlp {
+void count_in_flight(int, int by) {
+  in_flight += by;
+  if (in_flight > most_in_flight) most_in_flight = in_flight;
+}
 int set_error(int code, const char *msg) {
   std::printf("error %d %s\n", code, msg);
   return code;
@@ -30,7 +35,9 @@ int main(int argc, char **argv) {
   pdlp_mlp *net = nullptr;
   int written = 1;
   auto show = [&](const char *what, int rc) {
-    std::printf("%s %d pinned %d streams %d written %d\n", what, rc, n_pinned, n_streams, written);
+    std::printf("%s %d pinned %d streams %d written %d in_flight %d left %d\n", what, rc, n_pinned, n_streams, written,
+                most_in_flight, in_flight);
+    most_in_flight = 0;
   };
   show("create", pdlp_mlp_create(&net, in, hid, out, batch, nullptr));
   std::vector<float> X(300 * in, 1.0f);

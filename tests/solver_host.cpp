@@ -147,6 +147,12 @@ int main(int argc, char **argv) {
     show("run_b", pdlp_run_periods(b, 1));
     pdlp_destroy(a);
     show("run_b", pdlp_run_periods(b, 1));
+    show("poll_b", pdlp_poll(b, &st, &it));
+    {
+      const pdlp::InFlight batch(0);  // a batched solve or a network's call under way
+      show("run_b", pdlp_run_periods(b, 1));
+    }
+    show("run_b", pdlp_run_periods(b, 1));
     plan_cluster = true;  // a cluster leaves room: always its own launch
     pdlp_solver *c = create();
     show("begin_c", pdlp_begin(c, nullptr, nullptr, 1e-6, 100));

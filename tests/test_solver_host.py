@@ -94,7 +94,8 @@ def test_several_solvers_share_the_gpu_as_step_kernels(exe):
                    ("finish_a", 2, 2), ("run_b", 2, 3), ("poll_b", 2, 3),  # b alone
                    ("run_a", 2, 4), ("run_b", 3, 4),                     # a alone, then both
                    ("run_b", 3, 5),                                      # a destroyed
-                   ("begin_c", 3, 6), ("run_c", 3, 7)]                   # a cluster beside b
+                   ("poll_b", 3, 5), ("run_b", 4, 5), ("run_b", 4, 6),   # beside a batch, then alone
+                   ("begin_c", 4, 7), ("run_c", 4, 8)]                   # a cluster beside b
 
 
 @pytest.mark.parametrize("resident,small,large", [(152, 60, 40), (100, 60, 40), (40, 60, 40), (16, 60, 40), (20, 30, 1),
@@ -106,6 +107,7 @@ def test_a_batch_fits_its_grid_to_the_stream(batch_exe, resident, small, large):
     create, solve = _run(batch_exe, resident, small, large)
     assert create[1] == P.OK and solve[1] == P.OK
     assert solve[2]["grid"] == create[2]["grid"] > 0
+    assert create[2]["in_flight"] == solve[2]["in_flight"] == 1 and create[2]["left"] == solve[2]["left"] == 0
     if large:
         assert resident / 4 < create[2]["grid"] <= resident or create[2]["grid"] == 4 <= resident
     else:
@@ -118,6 +120,7 @@ def test_page_locked_chunks_come_where_a_large_pageable_prediction_pays_for_them
     assert [(r[0], r[2]["pinned"], r[2]["streams"]) for r in rows] == [
         ("create", 0, 1), ("small", 0, 1), ("locked", 0, 1), ("written", 0, 1), ("first", 0, 1), ("second", 1, 9),
         ("batches", 1, 9), ("big", 1, 10), ("written", 1, 10), ("once", 2, 18)]
+    assert [r[2]["in_flight"] for r in rows] == [0, 1, 1, 1, 1, 1, 1, 0, 1, 1] and rows[-1][2]["left"] == 0
 
 
 def test_predictions_without_page_locked_memory(mlp_exe):
