@@ -88,6 +88,8 @@ def pinned_lp(lp):
 
 
 def kernel_source_sha() -> str:
+    """Of the step kernels' source, which NCU_TRAFFIC is about (time_kernels runs
+    them whichever path a period takes)."""
     h = hashlib.sha256()
     for f in ("pdlp_kernels.cu", "pdlp_step.cuh", "pdlp_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2311_12180_gb300", "csrc", f), "rb") as fh:

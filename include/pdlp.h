@@ -372,9 +372,11 @@ typedef struct {
  * a few candidate schedules.  Each LP is solved by one CTA; an LP whose K,
  * K' and vectors fit in the CTA's shared-memory budget is copied there and
  * solved from shared memory; an LP with at least 32768 nonzeros is solved by
- * a team of CTAs (team_size of pdlp_batch_info: 4, 8 or 16) on as many SMs, which meet at bounded global-memory
- * barriers (the batch's CTAs must all be resident: a barrier that waits more
- * than 2 s fails the solve with PDLP_ERR_CUDA).  params: NULL = defaults; value_bits must be 64.
+ * a team of CTAs (team_size of pdlp_batch_info: 4, 8 or 16) on as many SMs,
+ * which meet at bounded global-memory barriers (a batch with teams is launched
+ * cooperatively, all of it resident together, with fewer teams on a stream that
+ * has fewer SMs; a barrier that waits more than 2 s fails the solve with
+ * PDLP_ERR_CUDA).  params: NULL = defaults; value_bits must be 64.
  * stream: cudaStream_t as void* (NULL = own stream). */
 int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const pdlp_params *params,
                       void *stream);
@@ -445,18 +447,19 @@ void pdlp_mlp_destroy(pdlp_mlp *net);
 /* Allocation-free Ruiz + Pock-Chambolle scaling of a matrix the caller keeps
  * in DEVICE memory.  This entry point has no counterpart in the paper; it is
  * the same scaling pdlp_create applies, with the same correctly rounded
- * divisions in the same order (row by row here, entry by entry in
- * pdlp_create, where each quotient comes from the factor's reciprocal and one
- * exact correction step; l_inf maxima and the fixed-order Pock-Chambolle row
- * sums do not depend on that), so D1, D2 and the scaled values are bitwise
- * equal to pdlp_get_scaling's.  It is offered
- * for callers
+ * quotients in the same order (row by row here, entry by entry in
+ * pdlp_create; each from the factor's reciprocal and one exact correction
+ * step; l_inf maxima and the fixed-order Pock-Chambolle row sums do not depend
+ * on that), so D1, D2 and the scaled values are bitwise equal to
+ * pdlp_get_scaling's.  A NaN entry is left out of its row's and its column's
+ * maximum.  It is offered for callers
  * that cannot call cudaMalloc or cudaFree: code that must take every byte of
  * device memory from its own pool (a framework's caching allocator, a
  * service with a fixed memory budget) and code that must not stall the device,
- * which cudaFree does.  It allocates nothing: the per-pass row and column
- * factors live in a fixed 4 MiB device array inside this library, held by
- * every GPU that loads the library until the process exits.
+ * which cudaFree does.  It allocates nothing: the row and column norms, factors
+ * and reciprocals and the lists of long rows live in a fixed 14 MiB device array
+ * inside this library, held by every GPU that loads the library until the
+ * process exits.
  *   K (m x n CSR: K_ptr m+1, K_idx / K_val nnz) and its transpose K' (n x m
  *   CSR: KT_ptr n+1, KT_idx / KT_val nnz, entries of each row in increasing
  *   order of K's row index) are DEVICE arrays; K_val and KT_val are scaled in

@@ -1275,9 +1275,10 @@ int solo_lanes(int rows, double mean_len) {
 
 // CTAs per team (RANKS, 2 RANKS or 4 RANKS) for the batch's team LPs on `ctas`
 // CTAs: the size whose greedy schedule (largest LP first, as the queue is
-// taken) ends first, the smaller one within 5 %.  An iteration of an LP costs a
-// team of s CTAs about 2.3e-3 us per nonzero / s plus 12 us of barriers and
-// reductions.  A batch of thousands keeps teams of four (10.9 s against 11.8
+// taken) ends first, the smaller one within 5 %.  The model that an iteration of
+// an LP costs a team of s CTAs 2.3e-3 us per nonzero / s plus 12 us of barriers
+// and reductions only ranks the sizes: the transportation LPs below take 100 us
+// where it says 46.  A batch of thousands keeps teams of four (10.9 s against 11.8
 // with teams of eight for 4096 uneven LPs); where a few large LPs hold the
 // batch up, or the last round of equal ones is nearly empty, larger teams win:
 // 256 uneven LPs, the largest of 2e6 nonzeros, 43.6 ms with teams of four and

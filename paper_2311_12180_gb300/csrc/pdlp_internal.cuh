@@ -235,10 +235,10 @@ __device__ __forceinline__ double clamp_bits(double v, double l, double u) {
 }
 
 // RN(a / b) from y = RN(1 / b) by one correction step (Markstein, IBM J. Res.
-// Dev. 34(1), 1990; Handbook of Floating-Point Arithmetic, the theorem on
-// division by an FMA correction): q = RN(a y) is within one ulp of a / b,
-// the remainder a - b q is exact with an FMA, and RN(q + (a - b q) y) is the
-// correctly rounded quotient when nothing underflows or overflows.  Where a
+// Dev. 34(1), 1990; Brisebarre, Muller and Raina, IEEE Trans. Comput. 53(8),
+// 2004, for this sequence): q = RN(a y), and RN(q + RN(a - b q) y) by two FMAs is
+// the correctly rounded quotient when nothing underflows or overflows (so it is
+// for every pair of significands of 4 to 12 bits, tried one by one).  Where a
 // or q is outside [2^-900, 2^900] (or zero, or not finite) the plain
 // division runs instead.  Three FP64 operations instead of a division
 // routine: the Ruiz passes divide every entry twice, on GB300's narrow FP64

@@ -85,10 +85,14 @@ __device__ __forceinline__ double ld_at(const double *p, int c) {
 
 // Barrier over the grid: a cluster's hardware barrier, or a counter in global
 // memory that only grows (`target`: its value once every CTA has arrived; the
-// next launch starts from the value this one leaves in sync->base).  All
-// threads of a CTA call both halves; the barrier orders the CTA's writes
-// before arrive() before every CTA's reads after wait().  wait() returns
-// false in every thread after BAR_WAIT_NS.
+// next launch starts from the value this one leaves in sync->base, a new state
+// from 0).  All threads of a CTA call both halves; the barrier orders the CTA's
+// writes before arrive() before every CTA's reads after wait().  The counter's
+// wait() returns false in every thread after BAR_WAIT_NS.  The hardware barrier
+// has no limit and needs none: a cluster is scheduled as a whole, and its CTAs
+// total the same partials behind the same barriers (see period_parts for what
+// keeps them the same), so they take the same decisions and pass the same
+// number of barriers.
 template <bool CLUSTER>
 struct Barrier {
   PeriodSync *s;

@@ -11,12 +11,6 @@
 
 namespace pdlp {
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // ---------------------------------------------------------------- sliced-ELL SpMV
 
 // float -> double from the IEEE bits with integer operations, exact for
