@@ -1639,7 +1639,7 @@ int pdlp_batch_create(pdlp_batch **out, int32_t count, const pdlp_lp *lps, const
     I.sk = team[i] ? lanes_for(mean_k[i], 4.0) : solo_lanes(I.m, mean_k[i]);
     I.st = team[i] ? lanes_for(mean_t[i], 4.0) : solo_lanes(I.n, mean_t[i]);
   }
-  const InFlight busy(b->device);
+  const InFlight busy(b->device, true);
   const double cands[3] = {4.0, 8.0, 16.0};
   auto lanes_of = [&](int i, double target, int *gk, int *gt) {
     const Inst &I = b->h_inst[i];
@@ -1720,7 +1720,7 @@ int pdlp_batch_solve(pdlp_batch *b, const double *x0, const double *y0, double t
   if (!b) return set_error(PDLP_ERR_INVALID, "pdlp_batch_solve: batch is NULL");
   if (!(tol >= 0.0) || max_iter < 1) return set_error(PDLP_ERR_INVALID, "pdlp_batch_solve: need tol >= 0, max_iter >= 1");
   BCK(cudaSetDevice(b->device));
-  const InFlight busy(b->device);
+  const InFlight busy(b->device, true);
   const double t0 = now_ms();
   cudaStream_t st = b->stream;
   Params p{};

@@ -61,23 +61,27 @@ struct Layout {
 };
 
 // Solvers of each device that have work enqueued which the host has not yet
-// waited for, and batched solves and network calls under way
-// (count_in_flight).  A whole-GPU period holds every SM, so solvers on several streams
-// would take turns, where the step kernels of small LPs share the GPU: four LPs
-// of 1e5 nonzeros take 7.9 us an iteration each as step kernels and 14.7 as
-// whole-GPU periods (alone 29.7 and 15.1), sixteen 3.1 and 14.8; two of 1e6
-// 23.7 and 30.2; and a batch on some of the SMs would keep it waiting to the
-// batch's end.  So such a period runs while its solver is the only one; its
-// results are the step kernels' bits, whichever run.  (A cluster leaves room
-// for eight others: sixteen solvers of 2e4 nonzeros take 1.6 us, 2.7 as step
-// kernels.)
-std::atomic<int> g_in_flight[64];
+// waited for, and batched solves and network calls under way (all, and the
+// batched solves among them: their kernels hold their SMs to the end).  A
+// whole-GPU period holds every SM, so solvers on several streams would take
+// turns, where the step kernels of small LPs share the GPU: four LPs of 1e5
+// nonzeros take 7.9 us an iteration each as step kernels and 14.7 as whole-GPU
+// periods (alone 29.7 and 15.1), sixteen 3.1 and 14.8; two of 1e6 23.7 and 30.2.
+// So such a period runs while its solver is the only one; its results are the
+// step kernels' bits, whichever run.  A cluster leaves room for eight others
+// (sixteen solvers of 2e4 nonzeros take 1.6 us, 2.7 as step kernels) and for
+// other kernels, but beside a batch of 60 to 140 CTAs no GPC has sixteen SMs for
+// it, and 2000 iterations wait for the batch's end: 178 ms, 35 as step kernels.
+std::atomic<int> g_in_flight[64], g_batches[64];
 
 }  // namespace
 
 int pdlp::set_error(int code, const char *msg) { return fail(code, msg ? msg : ""); }
 
-void pdlp::count_in_flight(int device, int by) { g_in_flight[device % 64] += by; }
+void pdlp::count_in_flight(int device, int by, bool batch) {
+  g_in_flight[device % 64] += by;
+  if (batch) g_batches[device % 64] += by;
+}
 
 struct pdlp_solver {
   int32_t m = 0, n = 0, n_eq = 0;
@@ -271,7 +275,8 @@ int try_period(pdlp_solver *s, int max_trials, bool *done) {
   if (capture != cudaStreamCaptureStatusNone)
     return fail(PDLP_ERR_CUDA, "a check period cannot be enqueued on a stream under capture");
   mark_in_flight(s, true);
-  if (!s->period.ctas || (!s->period.cluster && g_in_flight[s->device % 64] > 1)) return PDLP_OK;
+  const int d = s->device % 64;
+  if (!s->period.ctas || (s->period.cluster ? g_batches[d] > 0 : g_in_flight[d] > 1)) return PDLP_OK;
   const cudaError_t e = launch_period(s->period, s->K, s->KT, s->V, s->st, max_trials, s->stream);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
       e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration) {

@@ -205,13 +205,14 @@ cudaError_t kernels_init();  // one-time kernel attributes
 // Records `msg` as the calling thread's pdlp_last_error() and returns `code`.
 int set_error(int code, const char *msg);
 
-// Work on a device that whole-GPU periods should not wait for or hold up
+// Work on a device that one-launch periods should not wait for or hold up
 // (pdlp_capi.cu): one more or one less.
-void count_in_flight(int device, int by);
+void count_in_flight(int device, int by, bool batch = false);
 struct InFlight {
   int device;
-  explicit InFlight(int d) : device(d) { count_in_flight(device, 1); }
-  ~InFlight() { count_in_flight(device, -1); }
+  bool batch;
+  explicit InFlight(int d, bool b = false) : device(d), batch(b) { count_in_flight(device, 1, batch); }
+  ~InFlight() { count_in_flight(device, -1, batch); }
   InFlight(const InFlight &) = delete;
   InFlight &operator=(const InFlight &) = delete;
 };

@@ -17,7 +17,7 @@ extern const void *page_locked;
 
 static int in_flight = 0, most_in_flight = 0;
 namespace pdlp {
-void count_in_flight(int, int by) {
+void count_in_flight(int, int by, bool) {
   in_flight += by;
   if (in_flight > most_in_flight) most_in_flight = in_flight;
 }

@@ -149,13 +149,19 @@ int main(int argc, char **argv) {
     show("run_b", pdlp_run_periods(b, 1));
     show("poll_b", pdlp_poll(b, &st, &it));
     {
-      const pdlp::InFlight batch(0);  // a batched solve or a network's call under way
+      const pdlp::InFlight call(0);  // a network's call under way
       show("run_b", pdlp_run_periods(b, 1));
     }
     show("run_b", pdlp_run_periods(b, 1));
     plan_cluster = true;  // a cluster leaves room: always its own launch
     pdlp_solver *c = create();
     show("begin_c", pdlp_begin(c, nullptr, nullptr, 1e-6, 100));
+    show("run_c", pdlp_run_periods(c, 1));
+    {
+      const pdlp::InFlight batch(0, true);  // but not beside a batch
+      show("run_c", pdlp_run_periods(c, 1));
+      show("begin_c", pdlp_begin(c, nullptr, nullptr, 1e-6, 100));
+    }
     show("run_c", pdlp_run_periods(c, 1));
     pdlp_destroy(b);
     pdlp_destroy(c);

@@ -94,8 +94,9 @@ def test_several_solvers_share_the_gpu_as_step_kernels(exe):
                    ("finish_a", 2, 2), ("run_b", 2, 3), ("poll_b", 2, 3),  # b alone
                    ("run_a", 2, 4), ("run_b", 3, 4),                     # a alone, then both
                    ("run_b", 3, 5),                                      # a destroyed
-                   ("poll_b", 3, 5), ("run_b", 4, 5), ("run_b", 4, 6),   # beside a batch, then alone
-                   ("begin_c", 4, 7), ("run_c", 4, 8)]                   # a cluster beside b
+                   ("poll_b", 3, 5), ("run_b", 4, 5), ("run_b", 4, 6),   # beside a network, then alone
+                   ("begin_c", 4, 7), ("run_c", 4, 8),                   # a cluster beside b
+                   ("run_c", 5, 8), ("begin_c", 5, 8), ("run_c", 5, 9)]  # beside a batch, then not
 
 
 @pytest.mark.parametrize("resident,small,large", [(152, 60, 40), (100, 60, 40), (40, 60, 40), (16, 60, 40), (20, 30, 1),
